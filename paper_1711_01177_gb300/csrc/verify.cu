@@ -5,14 +5,14 @@
 // distance of r against b's span - the fewest edits that turn r into some
 // substring of the span (Sellers' recurrence: free start and end in the
 // text).  A location "results in a mapping" when that distance is <= E.
-// One thread per location runs Myers' bit-vector form of the recurrence:
-// the vertical differences of one text column, for 64 read positions per
-// machine word, advance by a handful of word operations per text base.
-// Reads of more than 64 bases are split into 64-row blocks that exchange
-// only the horizontal difference at their boundary row (Myers, 1999,
-// "A fast bit-vector algorithm for approximate string matching based on
-// dynamic programming", Sec. 4).  The read's match masks are built once per
-// location from its bases; text bases are decoded from the 2-bit reference.
+// One thread per location runs Myers' bit-vector form of the recurrence
+// (Myers, 1999, "A fast bit-vector algorithm for approximate string matching
+// based on dynamic programming"): the vertical differences of one column of
+// the table, 32 or 64 rows per machine word, advance by a handful of word
+// operations per column.  Spans of up to 1,024 bases are the rows, the read's
+// bases the columns (verify_rows_kernel); for longer spans the read's bases
+// are the rows, in 64-row blocks that exchange only the horizontal difference
+// at their boundary row (Myers, Sec. 4; verify_kernel).
 //
 // grim_verify_stats: counts of passing / rejected locations with and
 // without a mapping, from which the paper's "false negative rate" (passing
@@ -143,6 +143,233 @@ verify_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int64_t n_bins, 
     if (flags) atomicOr(status, flags);
 }
 
+// ------------------------------------------------------------ rows = the span
+
+// The same distances with the roles swapped: the rows of the table are the
+// span's bases (W 32-bit words, W fixed by the bank's geometry), its columns
+// the read's.  Every lane then runs the same code whatever its read's length,
+// a column's fixed costs are paid once per read base instead of once per span
+// base, and reads of different lengths share a warp with no divergence but
+// their trip counts, which the CTA evens out by sorting its locations by
+// length.  Boundary: D[i][0] = 0 (free start in the span), D[0][j] = j (the
+// horizontal difference entering the top row is always +1); the answer is the
+// minimum of the last column, found once from its vertical differences.
+//
+// Bound: the integer (ALU) pipe, at 10 operations per word and read base.
+// The match mask of a word is one shared-memory load instead of two logic
+// operations: the four masks of every word lie in the CTA's shared memory,
+// word-major with one column per thread (no bank conflicts).
+// 1M locations, reads of 50-300 bases, spans of 556 bases: 2.07 ms, where the
+// read-as-rows kernels took 14.9 ms (three launches, each with the lanes of
+// the other lengths idle, and 24 selects and logic operations a word).
+constexpr int kRowThreads = 128;
+constexpr int kRowMaxTile = 512;  // locations sorted together
+
+// Bits 0, 2, .. 30 of x packed into the low 16.
+__device__ __forceinline__ uint32_t even_bits(uint32_t x) {
+    x &= 0x55555555u;
+    x = (x | (x >> 1)) & 0x33333333u;
+    x = (x | (x >> 2)) & 0x0F0F0F0Fu;
+    x = (x | (x >> 4)) & 0x00FF00FFu;
+    return (x | (x >> 8)) & 0xFFFFu;
+}
+
+// 32-bit word k of the packed reference (16 bases); bytes past its end read 0.
+__device__ __forceinline__ uint32_t packed_word(const uint8_t* __restrict__ ref2bit, int64_t nbytes, bool aligned,
+                                                int64_t k) {
+    const int64_t b = 4 * k;
+    if (aligned && b + 4 <= nbytes) return __ldg(reinterpret_cast<const uint32_t*>(ref2bit + b));
+    uint32_t v = 0;
+    for (int i = 0; i < 4; i++)
+        if (b + i < nbytes) v |= (uint32_t)__ldg(ref2bit + b + i) << (8 * i);
+    return v;
+}
+
+__device__ __forceinline__ uint32_t add_cc(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm volatile("add.cc.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t addc_cc(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm volatile("addc.cc.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// One read base: Pv / Mv (rows whose vertical difference is +1 / -1) advance
+// by a column.  eq(w): match mask of word w.
+template <int W, typename Eq>
+__device__ __forceinline__ void rows_step(uint32_t (&Pv)[W], uint32_t (&Mv)[W], Eq&& eq) {
+    uint32_t ph_below = 0x80000000u, mh_below = 0;  // D[0][j] - D[0][j-1] = +1
+#pragma unroll
+    for (int w = 0; w < W; w++) {
+        const uint32_t e = eq(w), pv = Pv[w], mv = Mv[w];
+        const uint32_t a = e & pv;
+        const uint32_t s = w == 0 ? add_cc(a, pv) : addc_cc(a, pv);
+        const uint32_t xv = e | mv;
+        const uint32_t xh = (s ^ pv) | e;
+        const uint32_t ph = mv | ~(xh | pv);
+        const uint32_t mh = pv & xh;
+        const uint32_t phs = __funnelshift_l(ph_below, ph, 1);
+        const uint32_t mhs = __funnelshift_l(mh_below, mh, 1);
+        ph_below = ph;
+        mh_below = mh;
+        Pv[w] = mhs | ~(xv | phs);
+        Mv[w] = phs & xv;
+    }
+}
+
+template <int W>
+struct RowsSmem {
+    uint32_t eq[4][W][kRowThreads];  // match masks per base code, one column per thread
+    int16_t walk[256];               // four vertical differences (P nibble | M nibble << 4): min prefix << 8 | sum
+    uint16_t order[kRowMaxTile];     // the tile's locations, longest reads first
+    uint32_t count[64];              // by length class
+    int next;                        // first chunk of `order` not yet taken
+};
+
+// Locations [tile * blockIdx.x, ...): `tile` of them per CTA.  SPANs of at
+// most 32 W bases, reads of at most 64 kVerifyMaxBlocks.
+template <int W>
+__global__ void __launch_bounds__(kRowThreads)
+verify_rows_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int64_t n_bins, int bin_len, int overlap,
+                   const uint8_t* __restrict__ reads, const int64_t* __restrict__ read_offsets, int64_t n_reads,
+                   const uint32_t* __restrict__ loc_read, const uint32_t* __restrict__ loc_bin, int64_t n_loc,
+                   int tile, uint16_t* __restrict__ dist, uint32_t* __restrict__ status) {
+    extern __shared__ __align__(16) uint8_t rows_smem_raw[];
+    RowsSmem<W>& sm = *reinterpret_cast<RowsSmem<W>*>(rows_smem_raw);
+    const int t = threadIdx.x, lane = t & 31;
+    const int64_t i0 = (int64_t)blockIdx.x * tile;
+    const int n = (int)(n_loc - i0 < tile ? n_loc - i0 : tile);
+    if (t < 64) sm.count[t] = 0;
+    if (t == 0) sm.next = 0;
+    for (int x = t; x < 256; x += kRowThreads) {
+        int d = 0, mn = 0;
+        for (int k = 0; k < 4; k++) {
+            d += ((x >> k) & 1) - ((x >> (4 + k)) & 1);
+            mn = d < mn ? d : mn;
+        }
+        sm.walk[x] = (int16_t)((mn << 8) | (d & 0xFF));
+    }
+    __syncthreads();
+
+    // the tile's locations by read length (64 classes of 8 bases, longest
+    // first); one that cannot be scored is answered here
+    uint32_t flags = 0;
+    int cls[kRowMaxTile / kRowThreads];
+#pragma unroll
+    for (int k = 0; k < kRowMaxTile / kRowThreads; k++) {
+        const int i = k * kRowThreads + t;
+        cls[k] = -1;
+        if (i >= n) continue;
+        const uint32_t r = loc_read[i0 + i], b = loc_bin[i0 + i];
+        int64_t L = -1;
+        if ((int64_t)r < n_reads && (int64_t)b < n_bins) {
+            const int64_t ro = read_offsets[r], re = read_offsets[r + 1];
+            L = re >= ro ? re - ro : -1;
+        }
+        if (L < 0 || L > 64 * kVerifyMaxBlocks) {
+            flags |= (int64_t)b >= n_bins ? GRIM_FLAG_BAD_BIN
+                     : L > 64 * kVerifyMaxBlocks ? GRIM_FLAG_LONG_READ : GRIM_FLAG_BAD_OFFSETS;
+            dist[i0 + i] = 0xFFFF;
+            continue;
+        }
+        cls[k] = 63 - (int)(L > 0 ? (L - 1) >> 3 : 0);
+        atomicAdd(&sm.count[cls[k]], 1u);
+    }
+    __syncthreads();
+    if (t < 32) {  // counts -> first places
+        const uint32_t c0 = sm.count[2 * lane], c1 = sm.count[2 * lane + 1];
+        uint32_t x = c0 + c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, x, o);
+            if (lane >= o) x += y;
+        }
+        sm.count[2 * lane] = x - c0 - c1;
+        sm.count[2 * lane + 1] = x - c1;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kRowMaxTile / kRowThreads; k++)
+        if (cls[k] >= 0) sm.order[atomicAdd(&sm.count[cls[k]], 1u)] = (uint16_t)(k * kRowThreads + t);
+    __syncthreads();
+    const int n_ok = (int)sm.count[63];  // every place handed out
+
+    const int64_t nbytes = (len + 3) >> 2;
+    const bool aligned = ((uintptr_t)ref2bit & 3) == 0;
+    while (true) {  // warps take 32 locations at a time
+        int c = 0;
+        if (lane == 0) c = atomicAdd(&sm.next, 32);
+        c = __shfl_sync(kFull, c, 0);
+        if (c >= n_ok) break;
+        if (c + lane < n_ok) {
+            const int64_t i = i0 + sm.order[c + lane];
+            const uint32_t r = loc_read[i];
+            const int64_t begin = (int64_t)loc_bin[i] * bin_len;
+            const int64_t end = begin + bin_len + overlap < len ? begin + bin_len + overlap : len;
+            const int S = (int)(end - begin);  // rows
+            const int64_t ro = read_offsets[r];
+            const int L = (int)(read_offsets[r + 1] - ro);
+
+            // the span's match masks
+            const int sh = 2 * (int)(begin & 15);
+            const int64_t k0 = begin >> 4;
+            uint32_t lo = packed_word(ref2bit, nbytes, aligned, k0);
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+                const uint32_t mid = packed_word(ref2bit, nbytes, aligned, k0 + 2 * w + 1);
+                const uint32_t hi = packed_word(ref2bit, nbytes, aligned, k0 + 2 * w + 2);
+                const uint32_t x0 = __funnelshift_r(lo, mid, sh), x1 = __funnelshift_r(mid, hi, sh);
+                lo = hi;
+                const uint32_t b0 = even_bits(x0) | (even_bits(x1) << 16);
+                const uint32_t b1 = even_bits(x0 >> 1) | (even_bits(x1 >> 1) << 16);
+                sm.eq[0][w][t] = ~(b0 | b1);
+                sm.eq[1][w][t] = b0 & ~b1;
+                sm.eq[2][w][t] = ~b0 & b1;
+                sm.eq[3][w][t] = b0 & b1;
+            }
+
+            uint32_t Pv[W], Mv[W];
+#pragma unroll
+            for (int w = 0; w < W; w++) Pv[w] = Mv[w] = 0;  // D[i][0] = 0
+            const uint8_t* rd = reads + ro;
+            uint32_t next = L > 0 ? __ldg(rd) : 0u;
+            for (int j = 0; j < L; j++) {
+                const uint32_t code = next;
+                if (j + 1 < L) next = __ldg(rd + j + 1);
+                if (code <= 3u) {
+                    const uint32_t* eq = &sm.eq[code][0][t];
+                    rows_step<W>(Pv, Mv, [&](int w) { return eq[w * kRowThreads]; });
+                } else {
+                    rows_step<W>(Pv, Mv, [](int) { return 0u; });  // matches nothing
+                }
+            }
+
+            // minimum of D[0..S][L]: rows past the span only go up
+            int cur = L, best = L;
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+                const int rows = S - 32 * w;
+                const uint32_t in = rows >= 32 ? 0xFFFFFFFFu : rows <= 0 ? 0u : (1u << rows) - 1u;
+                const uint32_t p = Pv[w] | ~in, m = Mv[w] & in;
+#pragma unroll
+                for (int q = 0; q < 8; q++) {
+                    const uint32_t x = ((p >> (4 * q)) & 15u) | (((m >> (4 * q)) & 15u) << 4);
+                    const int step = sm.walk[x];
+                    const int low = cur + (step >> 8);
+                    best = low < best ? low : best;
+                    cur += (int)(int8_t)step;
+                }
+            }
+            dist[i] = (uint16_t)best;  // <= L <= 512
+        }
+        __syncwarp();
+    }
+    flags = __reduce_or_sync(kFull, flags);
+    if (lane == 0 && flags) atomicOr(status, flags);
+}
+
 // counts: [0] passing, [1] passing without a mapping (dist > E),
 //         [2] rejected, [3] rejected with a mapping (a miss)
 __global__ void verify_stats_kernel(const uint8_t* __restrict__ pass, const uint16_t* __restrict__ dist,
@@ -169,6 +396,46 @@ __global__ void verify_stats_kernel(const uint8_t* __restrict__ pass, const uint
     }
 }
 
+struct VerifyArgs {
+    const uint8_t* ref2bit;
+    const uint8_t* reads;
+    const int64_t* read_offsets;
+    int64_t n_reads;
+    const uint32_t* loc_read;
+    const uint32_t* loc_bin;
+    int64_t n_loc;
+    uint16_t* dist;
+};
+
+template <int W>
+int launch_verify_rows(const grim_bank* bank, const VerifyArgs& a, cudaStream_t s) {
+    constexpr size_t smem = sizeof(RowsSmem<W>);
+    static DeviceCache per_sm_of[64];  // per device, like the attribute
+    const int slot = device_slot();
+    if (slot < 0) return GRIM_ENOTSUP;
+    if (per_sm_of[slot].load() == 0) {
+        if (smem > 48 * 1024)
+            GRIM_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem));
+        int b = 0;
+        GRIM_CUDA_TRY(
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, verify_rows_kernel<W>, kRowThreads, smem));
+        per_sm_of[slot].store(b > 0 ? b : 1);
+    }
+    // the largest tile that still gives every resident CTA several: a larger
+    // tile sorts better, more tiles leave a shorter last wave
+    const int64_t want = 4 * (int64_t)sm_count() * per_sm_of[slot].load();
+    int tile = kRowMaxTile;
+    while (tile > kRowThreads && a.n_loc < want * tile) tile >>= 1;
+    const int64_t blocks = (a.n_loc + tile - 1) / tile;
+    if (blocks > 0x7fffffff) return GRIM_ENOTSUP;
+    verify_rows_kernel<W><<<grim::fault_grid((unsigned)blocks), kRowThreads, smem, s>>>(
+        a.ref2bit, bank->len, bank->n_bins, bank->bin_len, bank->overlap, a.reads, a.read_offsets, a.n_reads,
+        a.loc_read, a.loc_bin, a.n_loc, tile, a.dist, bank->status);
+    GRIM_CUDA_TRY(cudaGetLastError());
+    return GRIM_OK;
+}
+
 }  // namespace
 }  // namespace grim
 
@@ -183,6 +450,21 @@ int grim_verify(const grim_bank* bank, const uint8_t* ref2bit, const uint8_t* re
     int rc = grim::check_device(bank);
     if (rc != GRIM_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
+    const grim::VerifyArgs a{ref2bit, reads, read_offsets, n_reads, loc_read, loc_bin, n_loc, dist};
+    // the span as rows, W words of 32: spans of up to 1,024 bases (8 to 65 KB
+    // of match masks per CTA; W rounded up to the next of a few sizes, at most
+    // a quarter more work than the span needs above 256 bases); longer spans
+    // the read as rows
+    const int64_t words = ((int64_t)bank->bin_len + bank->overlap + 31) / 32;
+    if (words <= 8) return grim::launch_verify_rows<8>(bank, a, s);
+    if (words <= 10) return grim::launch_verify_rows<10>(bank, a, s);
+    if (words <= 12) return grim::launch_verify_rows<12>(bank, a, s);
+    if (words <= 13) return grim::launch_verify_rows<13>(bank, a, s);
+    if (words <= 15) return grim::launch_verify_rows<15>(bank, a, s);
+    if (words <= 18) return grim::launch_verify_rows<18>(bank, a, s);
+    if (words <= 21) return grim::launch_verify_rows<21>(bank, a, s);
+    if (words <= 26) return grim::launch_verify_rows<26>(bank, a, s);
+    if (words <= 32) return grim::launch_verify_rows<32>(bank, a, s);
     const int64_t need = (n_loc + 255) / 256;
     const int64_t cap = (int64_t)grim::sm_count() * 16;
     const unsigned blocks = (unsigned)(need < cap ? need : cap);
