@@ -370,8 +370,8 @@ int grim_scan(const grim_bank* bank, const uint8_t* reads, const int64_t* read_o
  * it while serving.  Arguments, outputs and results are those of grim_scan.
  *
  * Its working memory is one array of GRIM_SCAN_NOALLOC_SCRATCH_BYTES
- * (64 MiB) compiled into the library: every GPU on which the library is
- * loaded holds it until the process exits.  A call needing more is
+ * (64 MiB, and 128 KiB of padding) compiled into the library: every GPU on
+ * which the library is loaded holds it until the process exits.  A call needing more is
  * rejected with GRIM_ESCRATCH before anything is enqueued; the need is
  * 256 + sum over c = 0 .. 3 of ceil(n_reads / (256 >> c)) * 256 * K / 2
  * bytes (K = max(256, 4^q)) plus two small index arrays per c, which allows

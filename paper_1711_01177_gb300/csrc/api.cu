@@ -386,7 +386,8 @@ int grim_scan_noalloc(const grim_bank* bank, const uint8_t* reads, const int64_t
     size_t scratch_bytes = 0;
     rc = grim::scan_noalloc_scratch(&scratch, &scratch_bytes);
     if (rc != GRIM_OK) return rc;
-    if (grim::scan_scratch_bytes(bank->q, n_reads) > scratch_bytes) return GRIM_ESCRATCH;
+    if (!grim::scan_noalloc_admits(bank->q, n_reads) || grim::scan_scratch_bytes(bank->q, n_reads) > scratch_bytes)
+        return GRIM_ESCRATCH;
     cudaStream_t s = (cudaStream_t)stream;
     if (n_reads == 0 || bin_begin == bin_end) {
         GRIM_CUDA_TRY(cudaMemsetAsync(n_pairs, 0, sizeof(int64_t), s));

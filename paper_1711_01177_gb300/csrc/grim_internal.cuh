@@ -113,6 +113,8 @@ int launch_gather_batches(const grim_bank* bank, const GatherArgs& a, const grim
                           unsigned long long* counter, cudaStream_t stream);
 
 size_t scan_scratch_bytes(int q, int64_t n_reads);
+// Whether grim_scan_noalloc takes that many reads (the header's formula).
+bool scan_noalloc_admits(int q, int64_t n_reads);
 
 // The autotuned launch shape for this bank's q on its device (defaults
 // when grim_autotune has not run).

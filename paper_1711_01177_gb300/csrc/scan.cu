@@ -20,36 +20,48 @@
 // accumulation is exact and the pass decision is bit-identical to counting
 // tokens one by one.  Reads whose counts stay below 4 (nearly all) take one
 // row; counts up to 15, 255 and 65,535 take 2, 4 and 8; the prep kernel packs
-// reads into tiles of 256 rows by digit class (256 x 1, 128 x 2, 64 x 4, 32 x 8).
+// reads into tiles of 192 rows by digit class (192 x 1, 96 x 2, 48 x 4, 24 x 8).
 //
 // Data flow per CTA (persistent, one per SM; a work item = one read tile x
 // one run of bin tiles):
-//   B   : the read tile's 256 digit rows x K/2 bytes, staged once per work
+//   B   : the read tile's 192 digit rows x K/2 bytes, staged once per work
 //         item in shared memory in the 128-byte-swizzled K-major layout;
 //   bank: tiles of 128 bin rows stream through a 4-deep shared-memory ring
 //         by 2-D TMA tensor copies (warp 0), 16-byte chunks swizzled across
 //         the banks so that the expanders' row reads never collide;
-//   A   : warps 2-5 (one thread per bin = per TMEM lane) mask 512 bits of
-//         their bin's row into 512 e2m1 values and store them straight into
-//         tensor memory (3 stages of 64 columns, 8 MMAs per stage) - the
-//         expanded operand never touches shared memory;
-//   MMA : warp 1 issues M=128 (bins) x N=256 (rows) x K=64 tcgen05.mma with A
+//   A   : warps 2-9, two groups of four taking the stages in turn (one thread
+//         per bin = per TMEM lane), mask 256 bits of their bin's row into 256
+//         e2m1 values and store them straight into tensor memory (3 stages of
+//         32 columns, 4 MMAs per stage) - the expanded operand never touches
+//         shared memory;
+//   MMA : warp 1 issues M=128 (bins) x N=192 (rows) x K=64 tcgen05.mma with A
 //         from TMEM, B from shared memory and the unit scale factors from
-//         TMEM, accumulating in one 256-column TMEM accumulator (at N=256 an
-//         MMA runs at the full rate whatever the commits and operand
-//         rotation around it; at N=128 those cost ~40%);
-//   out : warps 6-21, four per lane quadrant, each load a quarter of the
-//         tile's accumulator columns (64) with tcgen05.ld in one round and
-//         hand the accumulator back to the MMAs at once (with one
-//         accumulator, the MMAs wait for it), then recombine digits,
-//         compare with each read's threshold and append the rare passing
-//         (read, bin, sum) triples with warp-aggregated atomics.
+//         TMEM, into one of two 192-column TMEM accumulators in turn;
+//   out : warps 10-17, two per lane quadrant, each load half of the tile's
+//         accumulator columns with tcgen05.ld in two rounds, recombine
+//         digits, compare with each read's threshold and append the rare
+//         passing (read, bin, sum) triples with warp-aggregated atomics, while
+//         the MMAs of the next tile run into the other accumulator.
+// Why N = 192: tensor memory has 512 columns.  One N = 256 accumulator beside
+// the A stages leaves the tensor pipe idle while it is drained and handed
+// back (~1,700 cycles per 2,050 of MMAs); two of them would leave no room for
+// A; two of 192 (384) leave 32 columns for the scale factors and 96 for A.
+// Measured, 16,384 reads of 100 bases against 12.1M bins: one accumulator of
+// 256, MMAs issued under `lane == 0` 95.8 ms; two of 192 88.0; eight expander
+// and eight epilogue warps 70.9; MMAs issued by an elected lane 59.5 (6.8
+// PFLOP/s, ~2,180 cycles per 128 x 192 tile whose MMAs take 1,650: the rest is
+// the expanders and the epilogue sharing the schedulers).  Tried beside it: A
+// stages of 128 tokens 94; tiles of 176 rows with a fourth A stage 60.0; one
+// expander group 62.5-64; 4 or 16 epilogue warps 66.6 and 72.6; the next
+// round's accumulator columns loaded before the last one's comparisons 73.9
+// (spills).
 // Every wait is an mbarrier try_wait bounded by a time limit; on expiry the
 // CTA raises GRIM_FLAG_TIMEOUT, drains and frees its tensor memory.
 #include <cuda.h>  // CUtensorMap (encoded through the runtime's driver entry point)
 #include <cudaTypedefs.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "grim_internal.cuh"
 #include "tcgen05.cuh"
@@ -61,27 +73,35 @@ namespace grim {
 // of the library, for callers that cannot allocate device memory.  Host code
 // must not pass the name itself to a kernel (on the host it is a stand-in,
 // not a device address); scan_noalloc_scratch() looks the address up.
-static __device__ __align__(256) uint8_t g_scan_scratch[GRIM_SCAN_NOALLOC_SCRATCH_BYTES];
+// What it admits is the header's formula, in tiles of 256 rows; tiles of
+// kRowsTile rows pad the classes of the reads it admits by at most 18,176
+// bytes more than that, which the array holds on top.
+constexpr size_t kNoallocSlack = size_t(128) << 10;
+static __device__ __align__(256) uint8_t g_scan_scratch[GRIM_SCAN_NOALLOC_SCRATCH_BYTES + kNoallocSlack];
 
 // ------------------------------------------------------------ constants
 
-constexpr int kScanThreads = 704;   // 22 warps: TMA, MMA, 4 expand, 16 epilogue
-constexpr int kExpandWarp0 = 2;     // expander warps 2..5, one per TMEM lane quadrant
-constexpr int kEpilogueWarp0 = 6;   // epilogue warps 6..21: four per quadrant, each a quarter of the reads
-constexpr int kEpilogueWarps = 16;
-static_assert(kEpilogueWarp0 == kExpandWarp0 + 4 && kScanThreads == 32 * (kEpilogueWarp0 + kEpilogueWarps),
-              "warp roles: TMA, MMA, four expanders, the epilogue");
+constexpr int kScanThreads = 576;   // 18 warps: TMA, MMA, 8 expand, 8 epilogue
+constexpr int kExpandWarp0 = 2;     // expander warps 2..9: two groups, each one warp per TMEM lane quadrant
+constexpr int kExpandGroups = 2;
+constexpr int kEpilogueWarp0 = kExpandWarp0 + 4 * kExpandGroups;  // epilogue warps 10..17: two per quadrant
+constexpr int kEpilogueWarps = 8;
+constexpr int kEpilogueRounds = 2;  // rounds a warp loads its share of the accumulator in
+static_assert(kEpilogueRounds == 2, "scan_epilogue");
+static_assert(kScanThreads == 32 * (kEpilogueWarp0 + kEpilogueWarps), "warp roles: TMA, MMA, expanders, the epilogue");
 constexpr int kBinTile = 128;       // bins per MMA tile (M, TMEM lanes)
-constexpr int kRowsTile = 256;      // B rows per read tile (N)
+constexpr int kRowsTile = 192;      // B rows per read tile (N)
 constexpr int kBankStages = 4;
-constexpr int kAStages = 3;         // A stages in tensor memory, filled by alternate expander groups
-constexpr int kAccCol = 0;          // the accumulator: columns [0, 256)
-constexpr int kSfCol = 256;         // unit scale factors of A and B: columns [256, 288)
-constexpr int kACol = 288;          // A stages: 3 x 64 columns from 288
+constexpr int kAStages = 3;         // A stages in tensor memory
+constexpr int kAccStages = 2;       // accumulators: columns [0, 192) and [192, 384)
+constexpr int kSfCol = kAccStages * kRowsTile;  // unit scale factors of A and B: columns [384, 416)
+constexpr int kACol = kSfCol + 32;  // A stages: 3 x 32 columns from 416
 constexpr int kTmemCols = 512;
 constexpr int kPrepWarps = 8;
 constexpr int kNumClasses = 4;      // digit classes: 1, 2, 4, 8 base-4 digits
 constexpr int kMmaK = 64;           // e2m1 K elements per MMA (32 bytes of a row)
+constexpr int kStageTok = 256;      // tokens per A stage
+static_assert(kACol + kAStages * kStageTok / 8 <= kTmemCols, "tensor memory columns");
 
 __host__ __device__ constexpr int class_digits(int c) { return 1 << c; }
 __host__ __device__ constexpr int class_reads(int c) { return kRowsTile >> c; }
@@ -92,7 +112,7 @@ struct ScanGeo {
     static constexpr int kRowBytes = kRowWords * 4;
     static constexpr int kK = (1 << (2 * Q)) < 256 ? 256 : (1 << (2 * Q));  // padded token count
     static constexpr int kKBytes = kK / 2;                                   // a B row: two e2m1 per byte
-    static constexpr int kChunkTok = kK >= 512 ? 512 : kK;                   // tokens per A stage
+    static constexpr int kChunkTok = kStageTok;                              // tokens per A stage
     static constexpr int kACols = kChunkTok / 8;                              // TMEM columns per A stage
     static constexpr int kWordsPerChunk = kChunkTok / 32;                     // bank words per A stage
     static constexpr int kMmaPerChunk = kChunkTok / kMmaK;                    // MMAs per A stage
@@ -104,14 +124,14 @@ struct ScanGeo {
     // rows), none for 16-byte rows
     static constexpr uint32_t kSwzMask = kRowBytes >= 128 ? 7u : (kRowBytes >= 32 ? 1u : 0u);
     static_assert(kRowBytes * 8 <= kK, "a bank row fits the padded K");
-    static_assert(kKBytes % 128 == 0 && kACols <= 64, "B rows are whole 128-byte swizzle atoms");
+    static_assert(kKBytes % 128 == 0 && kK % kChunkTok == 0, "B rows are whole 128-byte swizzle atoms");
 };
 
 // Scratch written by the prep kernel and read by the scan kernel.
 struct ScanScratch {
     int32_t* class_count;  // [4] reads per digit class
     int32_t* work;         // [1] work-item counter
-    uint8_t* rows[kNumClasses];   // digit rows, tiles of 128 rows x K/2 bytes (e2m1)
+    uint8_t* rows[kNumClasses];   // digit rows, tiles of 192 rows x K/2 bytes (e2m1)
     int32_t* T[kNumClasses];      // thresholds per slot (INT_MAX: never passes)
     uint32_t* rid[kNumClasses];   // read index per slot
 };
@@ -258,7 +278,7 @@ struct ScanSmem {
     static constexpr size_t kTf = kT + 4 * kRowsTile;
     static constexpr size_t kRid = kTf + 4 * kRowsTile;
     static constexpr size_t kBars = kRid + 4 * kRowsTile;
-    static constexpr size_t kMisc = kBars + 8 * (2 * kBankStages + 2 * kAStages + 5);
+    static constexpr size_t kMisc = kBars + 8 * (2 * kBankStages + 2 * kAStages + 2 * kAccStages + 1);
     static constexpr size_t kTotal = kMisc + 64;
     static constexpr size_t kAlloc = kTotal + 1024;  // slack to align the base
 };
@@ -305,12 +325,11 @@ __device__ __forceinline__ void scan_emit(const ScanParams& P, const int* sums, 
     }
 }
 
-// Epilogue of one work item for reads with D base-4 digits (N = 256 / D
+// Epilogue of one work item for reads with D base-4 digits (N = 192 / D
 // reads per tile): thread = bin row = TMEM lane of its warp's quadrant; the
-// warp takes the GR = 64 / D reads from quarter * N/4, i.e. 64 accumulator
-// columns.  Column d*N + n holds the digit-d sum of read n (an exact
+// warp takes half of the reads in two rounds.  Column d*N + n holds the digit-d sum of read n (an exact
 // integer in f32); Sum = sum_d 4^d * column d*N + n.  The accumulator is
-// handed back as soon as the columns are in registers.
+// handed back as soon as the last round's columns are in registers.
 template <int D>
 __device__ __forceinline__ void scan_epilogue(const ScanParams& P, uint32_t tmem, uint64_t* acc_full,
                                               uint64_t* acc_empty, volatile int* abort_flag,
@@ -318,63 +337,61 @@ __device__ __forceinline__ void scan_epilogue(const ScanParams& P, uint32_t tmem
                                               const uint32_t* __restrict__ sRid, int valid_reads, int64_t bt0,
                                               int64_t bt1, uint32_t& acc_cnt) {
     constexpr int N = kRowsTile / D;
-    constexpr int GR = 64 / D;  // reads of this warp: 64, 32, 16, 8
+    constexpr int NW = N * 4 / kEpilogueWarps;                             // reads of this warp
+    constexpr int GR = (NW + kEpilogueRounds - 1) / kEpilogueRounds;       // of a round (the last may have fewer)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quad = warp & 3;
-    const int quarter = (warp - kEpilogueWarp0) >> 2;
+    const int share = (warp - kEpilogueWarp0) >> 2;
     const int m = quad * 32 + lane;
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-    const uint32_t col0 = tmem + lane_base + kAccCol;
-    const int n0 = quarter * GR;  // first read of this warp
     for (int64_t bt = bt0; bt < bt1; bt++) {
-        const uint32_t phb = acc_cnt & 1;
-        if (!mbar_wait_warp(acc_full, phb, abort_flag)) break;
+        const uint32_t sacc = acc_cnt % kAccStages, phb = (acc_cnt / kAccStages) & 1;
+        if (!mbar_wait_warp(&acc_full[sacc], phb, abort_flag)) break;
         tc_fence_after();
+        const uint32_t col0 = tmem + lane_base + sacc * kRowsTile;
         const int64_t b = P.bin_begin + bt * kBinTile + m;
         const bool bin_ok = b < P.bin_end;
-        uint32_t v[64];
+        auto one_round = [&](auto first_c) {
+            constexpr int kFirst = decltype(first_c)::value, G = NW - kFirst < GR ? NW - kFirst : GR;
+            const int n0 = share * NW + kFirst;  // first read of this round
+            uint32_t v[D * G];
 #pragma unroll
-        for (int d = 0; d < D; d++) tmem_ld<GR>(col0 + d * N + n0, v + d * GR);
-        tmem_wait_ld();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(acc_empty);
-        if (D == 1) {
-            // one digit: the accumulator is the sum; compare it with T in f32
-            uint32_t any = 0;
-            const float4* t4 = reinterpret_cast<const float4*>(sTf + n0);
-#pragma unroll
-            for (int i = 0; i < GR / 4; i++) {
-                const float4 t = t4[i];  // four thresholds in one shared load
-                any |= (uint32_t)(__uint_as_float(v[4 * i]) >= t.x) |
-                       (uint32_t)(__uint_as_float(v[4 * i + 1]) >= t.y) |
-                       (uint32_t)(__uint_as_float(v[4 * i + 2]) >= t.z) |
-                       (uint32_t)(__uint_as_float(v[4 * i + 3]) >= t.w);
+            for (int d = 0; d < D; d++) tmem_ld_cols<G>(col0 + d * N + n0, v + d * G);
+            tmem_wait_ld();
+            if (kFirst + G == NW) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[sacc]);
             }
-            if (__any_sync(kFull, bin_ok && any)) {
-                int sums[GR];
+            bool any = false;
+            int sums[G];
+            if constexpr (D == 1 && G % 4 == 0 && NW % 4 == 0 && GR % 4 == 0) {
+                // one digit: the accumulator is the sum; compare it with T in
+                // f32, four thresholds a shared load
+                const float4* t4 = reinterpret_cast<const float4*>(sTf + n0);
 #pragma unroll
-                for (int i = 0; i < GR; i++) sums[i] = (int)__uint_as_float(v[i]);
-                scan_emit<GR>(P, sums, n0, valid_reads, sT, sRid, b, bin_ok, lane);
+                for (int i = 0; i < G / 4; i++) {
+                    const float4 t = t4[i];
+                    any = any | (__uint_as_float(v[4 * i]) >= t.x) | (__uint_as_float(v[4 * i + 1]) >= t.y) |
+                          (__uint_as_float(v[4 * i + 2]) >= t.z) | (__uint_as_float(v[4 * i + 3]) >= t.w);
+                }
+                if (!__any_sync(kFull, bin_ok && any)) return;
+#pragma unroll
+                for (int i = 0; i < G; i++) sums[i] = (int)__uint_as_float(v[i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < G; i++) {
+                    sums[i] = 0;
+#pragma unroll
+                    for (int d = 0; d < D; d++) sums[i] += (int)__uint_as_float(v[d * G + i]) << (2 * d);
+                    any = any | (sums[i] >= sT[n0 + i]);
+                }
+                if (!__any_sync(kFull, bin_ok && any)) return;
             }
-        } else {
-            int acc[GR];
-#pragma unroll
-            for (int i = 0; i < GR; i++) {
-                acc[i] = 0;
-#pragma unroll
-                for (int d = 0; d < D; d++) acc[i] += (int)__uint_as_float(v[d * GR + i]) << (2 * d);
-            }
-            uint32_t any = 0;
-            const int4* t4 = reinterpret_cast<const int4*>(sT + n0);
-#pragma unroll
-            for (int i = 0; i < GR / 4; i++) {
-                const int4 t = t4[i];
-                any |= (uint32_t)(acc[4 * i] >= t.x) | (uint32_t)(acc[4 * i + 1] >= t.y) |
-                       (uint32_t)(acc[4 * i + 2] >= t.z) | (uint32_t)(acc[4 * i + 3] >= t.w);
-            }
-            if (__any_sync(kFull, bin_ok && any)) scan_emit<GR>(P, acc, n0, valid_reads, sT, sRid, b, bin_ok, lane);
-        }
+            scan_emit<G>(P, sums, n0, valid_reads, sT, sRid, b, bin_ok, lane);
+        };
+        one_round(std::integral_constant<int, 0>{});
+        one_round(std::integral_constant<int, GR>{});
         acc_cnt++;
     }
 }
@@ -396,8 +413,8 @@ __global__ void __launch_bounds__(kScanThreads, 1) scan_kernel(const __grid_cons
     uint64_t* a_full = bars + 2 * kBankStages;
     uint64_t* a_empty = a_full + kAStages;
     uint64_t* acc_full = a_empty + kAStages;
-    uint64_t* acc_empty = acc_full + 1;
-    uint64_t* drain_bar = acc_empty + 1;
+    uint64_t* acc_empty = acc_full + kAccStages;
+    uint64_t* drain_bar = acc_empty + kAccStages;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + S::kMisc);
     volatile int* s_item = reinterpret_cast<volatile int*>(smem + S::kMisc + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + S::kMisc + 8);
@@ -409,14 +426,16 @@ __global__ void __launch_bounds__(kScanThreads, 1) scan_kernel(const __grid_cons
     if (threadIdx.x == 0) {
         for (int i = 0; i < kBankStages; i++) {
             mbar_init(&bank_full[i], 1);
-            mbar_init(&bank_empty[i], 4);
+            mbar_init(&bank_empty[i], 4 * kExpandGroups);
         }
         for (int i = 0; i < kAStages; i++) {
             mbar_init(&a_full[i], 4);
             mbar_init(&a_empty[i], 1);
         }
-        mbar_init(acc_full, 1);
-        mbar_init(acc_empty, kEpilogueWarps);
+        for (int i = 0; i < kAccStages; i++) {
+            mbar_init(&acc_full[i], 1);
+            mbar_init(&acc_empty[i], kEpilogueWarps);
+        }
         mbar_init(drain_bar, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -506,21 +525,21 @@ __global__ void __launch_bounds__(kScanThreads, 1) scan_kernel(const __grid_cons
                 }
             }
         } else if (warp == 1) {
-            // ---- MMA issuer
-            if (lane == 0) {
-                for (int64_t bt = bt0; bt < bt1; bt++) {
-                    const uint32_t phb = acc_cnt & 1;
-                    if (!mbar_wait(acc_empty, phb ^ 1, abort_flag)) break;
+            // ---- MMA issuer: the whole warp waits, one elected lane issues
+            bool ok = true;
+            for (int64_t bt = bt0; ok && bt < bt1; bt++) {
+                const uint32_t sacc = acc_cnt % kAccStages, phb = (acc_cnt / kAccStages) & 1;
+                if (!mbar_wait_warp(&acc_empty[sacc], phb ^ 1, abort_flag)) break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem + sacc * kRowsTile;
+                for (int c = 0; c < G::kChunks; c++) {
+                    const uint32_t sa = a_cnt % kAStages, pha = (a_cnt / kAStages) & 1;
+                    if (!mbar_wait_warp(&a_full[sa], pha, abort_flag)) {
+                        ok = false;
+                        break;
+                    }
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem + kAccCol;
-                    bool ok = true;
-                    for (int c = 0; c < G::kChunks; c++) {
-                        const uint32_t sa = a_cnt % kAStages, pha = (a_cnt / kAStages) & 1;
-                        if (!mbar_wait(&a_full[sa], pha, abort_flag)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
+                    if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < G::kMmaPerChunk; kk++) {
                             const uint32_t a_tmem = tmem + kACol + sa * G::kACols + kk * 8;
@@ -532,16 +551,17 @@ __global__ void __launch_bounds__(kScanThreads, 1) scan_kernel(const __grid_cons
                                            (c | kk) != 0);
                         }
                         mma_commit(&a_empty[sa]);
-                        a_cnt++;
+                        if (c == G::kChunks - 1) mma_commit(&acc_full[sacc]);
                     }
-                    if (!ok) break;
-                    mma_commit(acc_full);
-                    acc_cnt++;
+                    __syncwarp();
+                    a_cnt++;
                 }
+                if (ok) acc_cnt++;
             }
         } else if (warp < kEpilogueWarp0) {
             // ---- expanders: thread = bin row = TMEM lane
             const int quad = warp & 3;
+            const uint32_t group = (uint32_t)(warp - kExpandWarp0) >> 2;  // takes every kExpandGroups-th stage
             const int m = quad * 32 + lane;
             const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
             for (int64_t bt = bt0; bt < bt1; bt++) {
@@ -552,17 +572,26 @@ __global__ void __launch_bounds__(kScanThreads, 1) scan_kernel(const __grid_cons
                 const uint32_t tile_off = (uint32_t)s * G::kBankTileBytes + (uint32_t)m * G::kRowBytes;
                 bool ok = true;
                 for (int c = 0; c < G::kChunks; c++, a_cnt++) {
+                    if (a_cnt % kExpandGroups != group) continue;
                     const uint32_t sa = a_cnt % kAStages, pha = (a_cnt / kAStages) & 1;
                     // this stage's bank words (rows shorter than the padded K read as 0)
                     constexpr int kVec = G::kWordsPerChunk / 4;
-                    uint4 bits[kVec];
+                    uint32_t v[kVec][16];  // 4 bank words -> 16 columns
 #pragma unroll
                     for (int u = 0; u < kVec; u++) {
                         const int wv = c * kVec + u;  // 16-byte vector of the row
                         const uint32_t a = tile_off + 16u * wv;  // unswizzled offset, then the TMA's pattern
                         const uint32_t off = a ^ (((a >> 7) & G::kSwzMask) << 4);
-                        bits[u] = (m < rows && 4 * wv < G::kRowWords) ? *reinterpret_cast<const uint4*>(sBank + off)
-                                                                      : make_uint4(0, 0, 0, 0);
+                        const uint4 bits = (m < rows && 4 * wv < G::kRowWords)
+                                               ? *reinterpret_cast<const uint4*>(sBank + off)
+                                               : make_uint4(0, 0, 0, 0);
+                        expand_word_fp4(bits.x, v[u]);
+                        expand_word_fp4(bits.y, v[u] + 4);
+                        expand_word_fp4(bits.z, v[u] + 8);
+                        expand_word_fp4(bits.w, v[u] + 12);
+                        // masked before the wait below, not after it
+#pragma unroll
+                        for (int i = 0; i < 16; i++) asm volatile("" : "+r"(v[u][i]));
                     }
                     if (!mbar_wait_warp(&a_empty[sa], pha ^ 1, abort_flag)) {
                         ok = false;
@@ -570,19 +599,8 @@ __global__ void __launch_bounds__(kScanThreads, 1) scan_kernel(const __grid_cons
                     }
                     tc_fence_after();
 #pragma unroll
-                    for (int u = 0; u < kVec; u += 2) {
-                        // 8 bank words -> 32 columns (4 per word)
-                        uint32_t v[32];
-                        expand_word_fp4(bits[u].x, v);
-                        expand_word_fp4(bits[u].y, v + 4);
-                        expand_word_fp4(bits[u].z, v + 8);
-                        expand_word_fp4(bits[u].w, v + 12);
-                        expand_word_fp4(bits[u + 1].x, v + 16);
-                        expand_word_fp4(bits[u + 1].y, v + 20);
-                        expand_word_fp4(bits[u + 1].z, v + 24);
-                        expand_word_fp4(bits[u + 1].w, v + 28);
-                        tmem_st32(tmem + lane_base + kACol + sa * G::kACols + u * 16, v);
-                    }
+                    for (int u = 0; u < kVec; u++)
+                        tmem_st16(tmem + lane_base + kACol + sa * G::kACols + u * 16, v[u]);
                     tmem_wait_st();
                     tc_fence_before();
                     __syncwarp();
@@ -625,7 +643,9 @@ __global__ void __launch_bounds__(kScanThreads, 1) scan_kernel(const __grid_cons
                 }
             }
         }
-        if (threadIdx.x == 32) {  // every MMA this thread issued has finished once drain_bar completes
+        // the lane that issued the MMAs (one warp's election always falls on
+        // the same lane): they have finished once drain_bar completes
+        if (warp == 1 && elect_one()) {
             mma_commit(drain_bar);
             const unsigned long long t0 = now_ns();
             while (!mbar_try_wait(drain_bar, 0) && now_ns() - t0 < kWaitLimitNs) {
@@ -764,15 +784,21 @@ int scan_noalloc_scratch(void** ptr, size_t* bytes) {
     return GRIM_OK;
 }
 
-size_t scan_scratch_bytes(int q, int64_t n_reads) {
+static size_t scratch_for_tiles(int q, int64_t n_reads, int rows) {
     const int64_t K = (int64_t(1) << (2 * q)) < 256 ? 256 : (int64_t(1) << (2 * q));  // e2m1: K / 2 bytes a row
     size_t total = 256;
     for (int c = 0; c < kNumClasses; c++) {
-        const int64_t tiles = (n_reads + class_reads(c) - 1) / class_reads(c);
-        total += (size_t)tiles * kRowsTile * (K / 2);
-        total += 2 * (((size_t)tiles * class_reads(c) * 4 + 255) & ~(size_t)255);
+        const int64_t reads = rows >> c, tiles = (n_reads + reads - 1) / reads;
+        total += (size_t)tiles * rows * (K / 2);
+        total += 2 * (((size_t)tiles * reads * 4 + 255) & ~(size_t)255);
     }
     return total;
+}
+
+size_t scan_scratch_bytes(int q, int64_t n_reads) { return scratch_for_tiles(q, n_reads, kRowsTile); }
+
+bool scan_noalloc_admits(int q, int64_t n_reads) {
+    return scratch_for_tiles(q, n_reads, 256) <= GRIM_SCAN_NOALLOC_SCRATCH_BYTES;
 }
 
 int launch_scan(const grim_bank* bank, const uint8_t* reads, const int64_t* read_offsets, int64_t n_reads,
