@@ -1,7 +1,7 @@
 // Bank build (Sec. 3.1): the 2-bit packed reference -> one 4^q-bit
 // existence bitvector per bin, bin-major in HBM.
 //
-// Main kernel (bank_build_lanes_kernel, q <= 5 and ordinary geometry): one
+// Main kernel (bank_build_lanes_kernel, q <= 5 and bins of 16-1,024 bases): one
 // thread per bin CORE.  Bin b's token starts are its core's bin_len starts
 // followed by the first e = overlap - q + 1 starts after it, i.e. J whole
 // following cores and a prefix of r = e mod bin_len starts of the one after
@@ -20,18 +20,21 @@
 // rows pass through shared memory once more so that each warp stores its
 // consecutive rows with whole 512-byte writes.
 //
-// Fallback kernels (q = 6, very long bins or overlaps, unaligned input): one
-// CTA owns a run of consecutive bins and keeps their rows in shared memory;
-// its threads walk every token start of the run's spans once and set the
-// token's bit in every bin of the run whose span holds it with a
-// shared-memory atomicOr; the rows then leave in 16-byte stores.
+// q = 6 and geometry the main kernel does not take: bank_build_tile_kernel,
+// the same P and R rows for a run of cores per CTA, row-major.
+//
+// Fallback kernel (bins or overlaps too long for either): one CTA owns a run
+// of consecutive bins and keeps their rows in shared memory; its threads walk
+// every token start of the run's spans once and set the token's bit in every
+// bin of the run whose span holds it with a shared-memory atomicOr; the rows
+// then leave in 16-byte stores.
 #include "grim_internal.cuh"
 
 namespace grim {
 
 constexpr int kBuildThreads = 256;
 constexpr int kBuildSmemBytes = 16384;    // bin rows per CTA
-constexpr int kBuildStageBytes = 32768;   // staged packed reference per CTA
+constexpr int kTileStageBytes = 16384;    // staged packed reference per CTA
 
 template <int Q>
 __global__ void __launch_bounds__(kBuildThreads)
@@ -77,97 +80,11 @@ bank_build_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bin_len,
     for (int i = threadIdx.x; i < nb * row4; i += blockDim.x) dst[i] = smem4[i];
 }
 
-// Fast path: the run's packed reference bytes are staged in shared memory,
-// and each thread rolls the token through a contiguous stretch of token
-// starts (two instructions per base) while tracking, without divisions, the
-// first and last bin whose span holds the current token.
-template <int Q>
-__global__ void __launch_bounds__(kBuildThreads)
-bank_build_staged_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bin_len, int overlap, int64_t n_bins,
-                         int bins_per_cta, uint32_t* __restrict__ bank) {
-    using G = Geo<Q>;
-    constexpr uint32_t kMask = (Q == 16) ? 0xffffffffu : ((1u << (2 * Q)) - 1u);
-    extern __shared__ uint4 smem4[];
-    uint32_t* sbits = reinterpret_cast<uint32_t*>(smem4);
-    const int64_t b0 = (int64_t)blockIdx.x * bins_per_cta;
-    const int nb = (int)((n_bins - b0) < bins_per_cta ? (n_bins - b0) : bins_per_cta);
-    const int row4 = G::kRowWords / 4;
-    uint32_t* sref = sbits + (size_t)bins_per_cta * G::kRowWords;  // packed reference, 16 bases per word
-
-    const int64_t p0 = b0 * (int64_t)bin_len;
-    int64_t pend = (b0 + nb) * (int64_t)bin_len + overlap;
-    if (pend > len) pend = len;
-    // packed bytes [4*word0, 4*ceil(pend/16)) of the reference, as words
-    const int64_t word0 = p0 >> 4;
-    const int64_t byte_end = (pend + 3) >> 2;
-    const int nwords = (int)(((pend + 15) >> 4) - word0);
-    for (int i = threadIdx.x; i < nb * row4; i += blockDim.x) smem4[i] = make_uint4(0, 0, 0, 0);
-    for (int i = threadIdx.x; i < nwords; i += blockDim.x) {
-        uint32_t v = 0;
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const int64_t byte = 4 * (word0 + i) + k;
-            if (byte < byte_end) v |= (uint32_t)__ldg(ref2bit + byte) << (8 * k);
-        }
-        sref[i] = v;
-    }
-    __syncthreads();
-
-    // token starts i in [p0, pend - Q], split into one stretch per thread
-    const int n_starts = (int)(pend - Q + 1 - p0);
-    if (n_starts > 0) {
-        const int per = (n_starts + blockDim.x - 1) / blockDim.x;
-        const int s0 = threadIdx.x * per;
-        const int s1 = min(n_starts, s0 + per);
-        if (s0 < s1) {
-            // bases stream from a one-word buffer: x = position - 16*word0
-            int x = (int)(p0 + s0 - 16 * word0);
-            uint32_t buf = sref[x >> 4] >> (2 * (x & 15));
-            int left = 16 - (x & 15);
-            auto next_base = [&]() -> uint32_t {
-                if (left == 0) {
-                    buf = sref[x >> 4];
-                    left = 16;
-                }
-                const uint32_t b = buf & 3u;
-                buf >>= 2;
-                --left;
-                ++x;
-                return b;
-            };
-            uint32_t tok = 0;
-#pragma unroll
-            for (int k = 0; k < Q - 1; k++) tok = (tok << 2) | next_base();
-            // bin bookkeeping for the first start, then incremental
-            const int64_t i_first = p0 + s0;
-            int64_t bhi = i_first / bin_len;                           // last bin with b*bin_len <= i
-            int64_t next_hi = (bhi + 1) * (int64_t)bin_len;           // i at which bhi grows
-            const int64_t need = i_first + Q - (int64_t)bin_len - overlap;
-            int64_t blo = need <= 0 ? 0 : (need + bin_len - 1) / bin_len;  // first bin with i+Q <= its span end
-            int64_t next_lo = blo * (int64_t)bin_len + bin_len + overlap - Q + 1;  // i at which blo grows
-            const int64_t b_last = b0 + nb - 1;
-            for (int rel = s0; rel < s1; rel++) {
-                const int64_t i = p0 + rel;
-                if (i == next_hi) { ++bhi; next_hi += bin_len; }
-                if (i == next_lo) { ++blo; next_lo += bin_len; }
-                tok = ((tok << 2) | next_base()) & kMask;
-                const uint32_t w = tok >> 5, m = 1u << (tok & 31);
-                const int lo = (int)((blo > b0 ? blo : b0) - b0);
-                const int hi = (int)((bhi < b_last ? bhi : b_last) - b0);
-                for (int b = lo; b <= hi; b++) atomicOr(&sbits[b * G::kRowWords + w], m);
-            }
-        }
-    }
-    __syncthreads();
-    uint4* dst = reinterpret_cast<uint4*>(bank + b0 * G::kRowWords);
-    for (int i = threadIdx.x; i < nb * row4; i += blockDim.x) dst[i] = smem4[i];
-}
-
-
 // ------------------------------------------------------------ lane per core
 
 constexpr int kLaneWarps = 4;                  // 128 cores per CTA
 constexpr int kLaneCores = kLaneWarps * 32;
+constexpr int kLaneMinBinLen = 16;
 constexpr int kLaneMaxBinLen = 1024;           // staged bases per core (two staging buffers)
 constexpr int kLaneMaxJ = 16;                  // whole following cores in a span (out_w >= 15)
 
@@ -248,13 +165,19 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Issues the copies of one warp tile's packed words (its 32 cores from c0 and
-// the first word after them) into the warp's staging buffer; words past the
+// Packed words that hold the bases of a warp tile (its 32 cores, starting
+// `first` bases into the first word) and the token tails after them.
+__host__ __device__ constexpr int lane_tile_words(int bin_len, int first) {
+    return (first + 32 * bin_len + 15) / 16 + 1;
+}
+
+// Issues the copies of the packed words of a warp tile whose first core
+// starts at base p0 into the warp's staging buffer; words past the
 // reference are zero-filled by the copy itself.
-__device__ __forceinline__ void stage_warp_tile(const uint8_t* __restrict__ ref2bit, int64_t nbytes, int64_t c0,
-                                                int wpc, uint32_t stage_s, int lane) {
-    const int total = 32 * wpc + 1;
-    const int64_t g0 = c0 * (int64_t)wpc;
+__device__ __forceinline__ void stage_warp_tile(const uint8_t* __restrict__ ref2bit, int64_t nbytes, int64_t p0,
+                                                int bin_len, uint32_t stage_s, int lane) {
+    const int total = lane_tile_words(bin_len, (int)(p0 & 15));
+    const int64_t g0 = p0 >> 4;
     if (4 * (g0 + total) <= nbytes) {  // the whole tile lies inside the reference
         const uint8_t* src = ref2bit + 4 * g0;
         for (int i = lane; i < total; i += 32) cp_async4(stage_s + 4u * (uint32_t)stage_pos(i), src + 4 * i, 4);
@@ -274,17 +197,19 @@ __device__ __forceinline__ void stage_warp_tile(const uint8_t* __restrict__ ref2
 // 32 - (J + 1) (the last J + 1 cores only complete their neighbours' rows),
 // so a warp never waits for another.  The next warp tile's reference words
 // are copied in while the current one is built.
-template <int Q>
+// WORDS: cores start at word boundaries (bin_len a multiple of 16); otherwise
+// each word of bases is funnelled together from two staged words (1 Gbp, q = 5:
+// bins of 255 bases 327 us as those of 256; 2,195 us before this form).
+template <int Q, bool WORDS>
 __global__ void __launch_bounds__(kLaneCores, 4)
-bank_build_lanes_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bin_len, int r_pref, int J,
+bank_build_lanes_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bin_len, int starts, int r_pref, int J,
                         int64_t n_bins, int64_t n_units, uint32_t* __restrict__ bank) {
     using LG = LaneGeo<Q>;
     constexpr int RW = LG::kRW;
     extern __shared__ uint4 lane_smem4[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int out_w = 32 - (J + 1);   // rows finished per warp tile
-    const int wpc = bin_len >> 4;     // packed words per core
-    const int stage_words = stage_pos(32 * wpc + 1) + 1;
+    const int stage_words = stage_pos(lane_tile_words(bin_len, 15)) + 1;
     const int64_t nbytes = (len + 3) >> 2;
 
     // rows: the P and R row sets of every warp, aligned so that the word
@@ -304,7 +229,7 @@ bank_build_lanes_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bi
 
     const int64_t stride = (int64_t)gridDim.x * kLaneWarps;
     int64_t unit = (int64_t)blockIdx.x * kLaneWarps + warp;
-    if (unit < n_units) stage_warp_tile(ref2bit, nbytes, unit * out_w, wpc, my_stage_s, lane);
+    if (unit < n_units) stage_warp_tile(ref2bit, nbytes, unit * out_w * bin_len, bin_len, my_stage_s, lane);
     cp_async_commit();
     // the row sets start zeroed; afterwards every read of them (the rows,
     // then the staged output) swaps in zeros, so no tile needs a clearing pass
@@ -315,21 +240,35 @@ bank_build_lanes_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bi
         const int buf = it & 1;
         const int64_t next = unit + stride;
         if (next < n_units)
-            stage_warp_tile(ref2bit, nbytes, next * out_w, wpc, my_stage_s + 4u * (uint32_t)(stage_words * (buf ^ 1)),
-                            lane);
+            stage_warp_tile(ref2bit, nbytes, next * out_w * bin_len, bin_len,
+                            my_stage_s + 4u * (uint32_t)(stage_words * (buf ^ 1)), lane);
         cp_async_commit();
         cp_async_wait<1>();  // this tile's words have landed (the next tile's may not)
         __syncwarp();
 
-        // token starts of this core: [0, n_lane) (clipped at the reference end)
+        // token starts of this core: [0, n_lane), `starts` of them (clipped at the reference end)
         {
             const int64_t left = len - Q + 1 - (c0 + lane) * (int64_t)bin_len;
-            const int n_lane = left <= 0 ? 0 : (left < bin_len ? (int)left : bin_len);
+            const int n_lane = left <= 0 ? 0 : (left < starts ? (int)left : starts);
             const uint32_t* st = my_stage + stage_words * buf;
-            const int g = lane * wpc;
-            uint32_t hi = reverse_bases(st[stage_pos(g)]);
-            for (int j = 0; j < wpc; j++) {
-                const uint32_t lo = reverse_bases(st[stage_pos(g + j + 1)]);
+            // the core's bases 16 j .. 16 j + 15, first base highest, in hi
+            const int o = WORDS ? lane * bin_len : (int)(c0 * bin_len & 15) + lane * bin_len;
+            const int g = o >> 4, sh = 2 * (o & 15);
+            uint32_t w1 = reverse_bases(st[stage_pos(g)]);
+            uint32_t hi = w1;
+            if (!WORDS) {
+                const uint32_t w0 = w1;
+                w1 = reverse_bases(st[stage_pos(g + 1)]);
+                hi = __funnelshift_l(w1, w0, sh);
+            }
+            const int groups = (bin_len + 15) >> 4;
+            for (int j = 0; j < groups; j++) {
+                uint32_t lo = reverse_bases(st[stage_pos(g + j + (WORDS ? 1 : 2))]);
+                if (!WORDS) {
+                    const uint32_t w2 = lo;
+                    lo = __funnelshift_l(w2, w1, sh);
+                    w1 = w2;
+                }
                 const int s0 = 16 * j;
                 const int split = r_pref - s0;  // starts below it go to P (uniform over the warp)
                 if (s0 + 16 <= n_lane) {
@@ -391,11 +330,12 @@ bank_build_lanes_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bi
 template <int Q>
 constexpr size_t lane_smem_bytes(int bin_len) {
     return (size_t)kLaneWarps * 2 * LaneGeo<Q>::kRowSetBytes + LaneGeo<Q>::kRowSetBytes +
-           (size_t)kLaneWarps * 2 * 4 * (size_t)(32 * (bin_len >> 4) + 1 + ((32 * (bin_len >> 4) + 1) >> 5) + 1);
+           (size_t)kLaneWarps * 2 * 4 *
+               (size_t)(lane_tile_words(bin_len, 15) + (lane_tile_words(bin_len, 15) >> 5) + 1);
 }
 
-template <int Q>
-static int launch_lanes(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s, int r_pref, int J) {
+template <int Q, bool WORDS>
+static int launch_lanes(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s, int starts, int r_pref, int J) {
     const int out_w = 32 - (J + 1);
     const int64_t n_units = (bank->n_bins + out_w - 1) / out_w;
     const size_t smem = lane_smem_bytes<Q>(bank->bin_len);
@@ -404,17 +344,149 @@ static int launch_lanes(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s,
     if (slot < 0) return GRIM_ENOTSUP;
     if (attr[slot].load() < (int)smem) {
         GRIM_CUDA_TRY(
-            cudaFuncSetAttribute(bank_build_lanes_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            cudaFuncSetAttribute(bank_build_lanes_kernel<Q, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr[slot].store((int)smem);
     }
     int per_sm = 0;
-    GRIM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bank_build_lanes_kernel<Q>, kLaneCores, smem));
+    GRIM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bank_build_lanes_kernel<Q, WORDS>, kLaneCores, smem));
     if (per_sm < 1) return GRIM_ENOTSUP;  // cannot happen below kLaneMaxBinLen
     int64_t blocks = (int64_t)sm_count() * per_sm;
     const int64_t need = (n_units + kLaneWarps - 1) / kLaneWarps;
     if (blocks > need) blocks = need;
-    bank_build_lanes_kernel<Q><<<grim::fault_grid((unsigned)blocks), kLaneCores, smem, s>>>(
-        ref2bit, bank->len, bank->bin_len, r_pref, J, bank->n_bins, n_units, bank->bits);
+    bank_build_lanes_kernel<Q, WORDS><<<grim::fault_grid((unsigned)blocks), kLaneCores, smem, s>>>(
+        ref2bit, bank->len, bank->bin_len, starts, r_pref, J, bank->n_bins, n_units, bank->bits);
+    GRIM_CUDA_TRY(cudaGetLastError());
+    return GRIM_OK;
+}
+
+// ------------------------------------------------------------ tile of cores
+
+// q = 6 (512-byte rows: the lane kernel's 32 KB of rows a warp leave an SM
+// four warps; 100 Mbp, 256 + 300: 274 us) and other geometry the lane kernel
+// does not take.  One CTA owns a run of consecutive
+// cores with their P and R rows (see the top) in shared memory, row-major:
+//   1. the run's packed bases are staged, first base highest;
+//   2. each thread sets the bits of 16 consecutive token starts of one core
+//      at a time (compile-time shifts of a 64-bit window, as above): once per
+//      token, in P or R, where the kernel before it set each token once per
+//      bin that holds it after walking the bins' bounds token by token;
+//   3. each thread ORs one 16-byte column of consecutive rows together and
+//      stores it.
+// Bound: shared-memory wavefronts (89% of the pipe's rate; the 32 ORs of a
+// warp hit random banks, about 3.5 to the busiest).  q = 6, 100 Mbp, 256 + 300:
+// 261 -> 97 us.
+template <int Q>
+struct TileGeo {
+    static constexpr int kRW = Geo<Q>::kRowWords;
+    static constexpr int kMaxCores = 16384 / (4 * kRW);  // 16 KB per row set
+    static constexpr int kVecs = kRW / 4;
+    // byte offset of a token's row word, as a mask on the token shifted right by 3
+    static constexpr uint32_t kWordMask = Q >= 3 ? (uint32_t)((1u << (2 * Q - 5)) - 1u) << 2 : 0u;
+};
+
+template <int Q, int T>
+__device__ __forceinline__ void tile_token_step(uint32_t hi, uint32_t lo, uint32_t base0, uint32_t base1, int split,
+                                                int lim) {
+    if constexpr (T < 16) {
+        constexpr int kShift = 64 - 2 * T - 2 * Q;
+        const uint32_t x = lane_window<Q, T>(hi, lo);
+        // the token's row word: x >> 3 (with the bases before it above)
+        uint32_t word = 0;
+        if constexpr (Q >= 3) {
+            static_assert(kShift + 3 < 64, "a shift within the window");
+            if constexpr (kShift + 3 >= 32) word = hi >> (kShift + 3 - 32);
+            else word = __funnelshift_r(lo, hi, kShift + 3);
+        }
+        if (T < lim) {
+            const uint32_t tok = Q < 3 ? (x & ((1u << (2 * Q)) - 1u)) : x;
+            red_or_shared((word & TileGeo<Q>::kWordMask) | (T < split ? base0 : base1),
+                          __funnelshift_l(0u, 1u, tok));  // 1 << (tok & 31)
+        }
+        tile_token_step<Q, T + 1>(hi, lo, base0, base1, split, lim);
+    }
+}
+
+template <int Q>
+__global__ void __launch_bounds__(kBuildThreads)
+bank_build_tile_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bin_len, int starts, int r_pref, int J,
+                       int cores, int64_t n_bins, uint32_t* __restrict__ bank) {
+    using G = TileGeo<Q>;
+    extern __shared__ uint4 tile_smem4[];
+    const int64_t b0 = (int64_t)blockIdx.x * (cores - J - 1);  // first core and first finished row
+    const int n_vec = 2 * cores * G::kVecs;
+    // P rows, then R rows, aligned so that a row's address and its word
+    // offsets share no bits; then the staged bases
+    const uint32_t raw = shared_addr(tile_smem4);
+    uint4* rows = tile_smem4 + (((raw + 4 * G::kRW - 1) & ~(uint32_t)(4 * G::kRW - 1)) - raw) / 16;
+    uint32_t* sref = reinterpret_cast<uint32_t*>(rows + n_vec);
+    for (int i = threadIdx.x; i < n_vec; i += kBuildThreads) rows[i] = make_uint4(0, 0, 0, 0);
+
+    const int64_t p0 = b0 * bin_len;
+    const int64_t word0 = p0 >> 4, nbytes = (len + 3) >> 2;
+    const int first = (int)(p0 & 15);
+    const int n_words = (first + cores * bin_len + 15) / 16 + 2;
+    const bool aligned = ((uintptr_t)ref2bit & 3) == 0;
+    for (int i = threadIdx.x; i < n_words; i += kBuildThreads) {
+        const int64_t byte = 4 * (word0 + i);
+        uint32_t v = 0;
+        if (aligned && byte + 4 <= nbytes) {
+            v = __ldg(reinterpret_cast<const uint32_t*>(ref2bit + byte));
+        } else {
+            for (int k = 0; k < 4; k++)
+                if (byte + k < nbytes) v |= (uint32_t)__ldg(ref2bit + byte + k) << (8 * k);
+        }
+        sref[i] = reverse_bases(v);
+    }
+    __syncthreads();
+
+    const int groups = (bin_len + 15) >> 4;  // of 16 token starts per core
+    const uint32_t rows_s = shared_addr(rows), set_bytes = (uint32_t)(cores * G::kRW * 4);
+    for (int i = threadIdx.x; i < cores * groups; i += kBuildThreads) {
+        const int core = i / groups, s0 = 16 * (i - core * groups);
+        const int64_t left = len - Q + 1 - (p0 + (int64_t)core * bin_len + s0);  // starts before the reference's end
+        int lim = starts - s0 < 16 ? starts - s0 : 16;  // none when it is not positive
+        if (left < lim) lim = left > 0 ? (int)left : 0;
+        const int o = first + core * bin_len + s0;
+        const int g = o >> 4, sh = 2 * (o & 15);
+        const uint32_t w0 = sref[g], w1 = sref[g + 1], w2 = sref[g + 2];
+        const uint32_t base0 = rows_s + (uint32_t)(core * G::kRW * 4);
+        tile_token_step<Q, 0>(__funnelshift_l(w1, w0, sh), __funnelshift_l(w2, w1, sh), base0, base0 + set_bytes,
+                              r_pref - s0, lim);
+    }
+    __syncthreads();
+
+    const int out = (int)(n_bins - b0 < cores - J - 1 ? n_bins - b0 : cores - J - 1);
+    const int r_off = cores * G::kVecs;
+    uint4* dst = reinterpret_cast<uint4*>(bank + b0 * G::kRW);
+    for (int i = threadIdx.x; i < out * G::kVecs; i += kBuildThreads) {
+        const int last = i + (J + 1) * G::kVecs;  // the same column, J + 1 rows on
+        uint4 v = rows[last];
+        for (int a = i; a < last; a += G::kVecs) {
+            const uint4 p = rows[a], r = rows[a + r_off];
+            v.x |= p.x | r.x;
+            v.y |= p.y | r.y;
+            v.z |= p.z | r.z;
+            v.w |= p.w | r.w;
+        }
+        dst[i] = v;
+    }
+}
+
+template <int Q>
+static int launch_tile(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s, int starts, int r_pref, int J,
+                       int cores, size_t smem) {
+    const int64_t blocks = (bank->n_bins + cores - J - 2) / (cores - J - 1);
+    if (blocks > 0x7fffffff) return GRIM_ENOTSUP;
+    static DeviceCache attr[64];  // per device: the largest size set so far
+    const int slot = device_slot();
+    if (slot < 0) return GRIM_ENOTSUP;
+    if (smem > 48 * 1024 && attr[slot].load() < (int)smem) {
+        GRIM_CUDA_TRY(
+            cudaFuncSetAttribute(bank_build_tile_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        attr[slot].store((int)smem);
+    }
+    bank_build_tile_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads, smem, s>>>(
+        ref2bit, bank->len, bank->bin_len, starts, r_pref, J, cores, bank->n_bins, bank->bits);
     GRIM_CUDA_TRY(cudaGetLastError());
     return GRIM_OK;
 }
@@ -422,35 +494,32 @@ static int launch_lanes(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s,
 template <int Q>
 static int launch_q(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s) {
     using G = Geo<Q>;
-    // lane-per-core kernel for q <= 5, bins of a multiple of 16 bases, an
-    // overlap that holds at least the last token of the core, word-aligned input
+    const int bl = bank->bin_len;
     const int64_t e = (int64_t)bank->overlap - Q + 1;  // token starts past the core
-    if (Q <= 5 && bank->bin_len % 16 == 0 && bank->bin_len <= kLaneMaxBinLen && e >= 0 &&
-        e / bank->bin_len <= kLaneMaxJ && ((uintptr_t)ref2bit & 3) == 0)
-        return launch_lanes<Q <= 5 ? Q : 5>(ref2bit, bank, s, (int)(e % bank->bin_len), (int)(e / bank->bin_len));
+    // an overlap shorter than a token (e < 0) leaves out the core's last -e
+    // starts; the row then is the core's own, all of it in P (J = -1)
+    const int64_t J = e >= 0 ? e / bl : -1;
+    const int r_pref = e >= 0 ? (int)(e % bl) : bl;
+    const int starts = e >= 0 ? bl : (bl + e > 0 ? (int)(bl + e) : 0);
+    if constexpr (Q <= 5) {
+        if (bl >= kLaneMinBinLen && bl <= kLaneMaxBinLen && J <= kLaneMaxJ && ((uintptr_t)ref2bit & 3) == 0)
+            return bl % 16 == 0 ? launch_lanes<Q, true>(ref2bit, bank, s, starts, r_pref, (int)J)
+                                : launch_lanes<Q, false>(ref2bit, bank, s, starts, r_pref, (int)J);
+    }
+    // a tile of cores, as many as 16 KB of rows and 16 KB of staged bases
+    // allow, at least half of whose rows are finished
+    const int64_t fit = (kTileStageBytes / 4 - 4) * 16 / bl;
+    const int64_t cores = fit < TileGeo<Q>::kMaxCores ? fit : TileGeo<Q>::kMaxCores;
+    if (cores > 0 && 2 * (J + 1) <= cores)
+        return launch_tile<Q>(
+            ref2bit, bank, s, starts, r_pref, (int)J, (int)cores,
+            (size_t)(2 * cores + 1) * G::kRowWords * 4 + 4 * (size_t)((cores * bl + 30) / 16 + 2));
     const int bins_per_cta = kBuildSmemBytes / (G::kRowWords * 4);
     const int64_t blocks = (bank->n_bins + bins_per_cta - 1) / bins_per_cta;
     if (blocks > 0x7fffffff) return GRIM_ENOTSUP;
-    const size_t smem_rows = (size_t)bins_per_cta * G::kRowWords * 4;
-    // staged path when a run's packed reference bytes fit beside its rows
-    const int64_t span = (int64_t)bins_per_cta * bank->bin_len + bank->overlap;
-    const int64_t stage = 4 * (span / 16 + 3);
-    if (stage <= kBuildStageBytes) {
-        const size_t smem = smem_rows + (size_t)((stage + 15) & ~15LL);
-        static DeviceCache attr[64];  // per device
-        const int slot = device_slot();
-        if (slot < 0) return GRIM_ENOTSUP;
-        if (!attr[slot].load() && smem > 48 * 1024) {
-            GRIM_CUDA_TRY(cudaFuncSetAttribute(bank_build_staged_kernel<Q>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            attr[slot].store(1);
-        }
-        bank_build_staged_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads, smem, s>>>(
-            ref2bit, bank->len, bank->bin_len, bank->overlap, bank->n_bins, bins_per_cta, bank->bits);
-    } else {
-        bank_build_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads, smem_rows, s>>>(
-            ref2bit, bank->len, bank->bin_len, bank->overlap, bank->n_bins, bins_per_cta, bank->bits);
-    }
+    bank_build_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads,
+                           (size_t)bins_per_cta * G::kRowWords * 4, s>>>(
+        ref2bit, bank->len, bank->bin_len, bank->overlap, bank->n_bins, bins_per_cta, bank->bits);
     GRIM_CUDA_TRY(cudaGetLastError());
     return GRIM_OK;
 }
