@@ -10,12 +10,14 @@
 //     location p of the seed at offset o votes for the bin whose core holds
 //     max(0, p - o); distinct bins are kept, the `cap` most voted when
 //     there are more (equal votes: the lower bin), ascending.  Per batch of
-//     reads: hits per read (warp per read) -> prefix sum -> votes expanded
-//     into scratch -> one CTA per read sorts its votes (stable LSD radix
-//     sort, in shared memory up to kDedupSmem votes, else in global
-//     scratch), finds the runs, applies the cap (binary search on the vote
-//     threshold) and compacts -> prefix sum of the kept counts -> copy into
-//     the CSR output.
+//     reads: hits per read (warp per read) -> prefix sum -> seed_fast_kernel:
+//     a group of threads per read fetches its seeds' locations, sorts the
+//     voted bins in shared memory and keeps the distinct ones; the few reads
+//     it cannot take (too many votes, votes piled into one region, more bins
+//     than the cap) are listed and go through votes in scratch -> one CTA per
+//     read that sorts them (bucket or stable LSD radix sort), finds the runs,
+//     applies the cap (binary search on the vote threshold) and compacts ->
+//     prefix sum of the kept counts -> copy into the CSR output.
 // After (Sec. 3.3, Fig. 4 steps 2-3): the Seed Location Checker turns the
 // filter's bitmask into the list of passing locations and the reference
 // segments the aligner receives.
@@ -233,40 +235,534 @@ __global__ void seed_hits_kernel(const uint32_t* __restrict__ idx_off, int k, co
     }
 }
 
-// The batch's votes: read r's bins at H[hit_off[r] - h0 ...] (warp per read;
-// seeds in order, each seed's locations spread over the lanes).
+// Quotient of any 32-bit n by a fixed divisor (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", 1994, fig. 4.1).
+struct FastDiv {
+    uint32_t mul;
+    int sh1, sh2;
+    explicit FastDiv(uint32_t d) {
+        int l = 0;
+        while (l < 32 && (uint64_t(1) << l) < d) l++;
+        mul = (uint32_t)(((uint64_t(1) << 32) * ((uint64_t(1) << l) - d)) / d + 1);
+        sh1 = l < 1 ? l : 1;
+        sh2 = l > 1 ? l - 1 : 0;
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t n) const {
+        const uint32_t t = __umulhi(mul, n);
+        return (t + ((n - t) >> sh1)) >> sh2;
+    }
+};
+
+// ---- the common case: a group of T threads per read, in shared memory
+//
+// The distinct bins come from a bitmap of the bin ids scaled to 32 V T bits
+// (T = 128, V = 24: 98,304): a vote that finds its bit clear is its cell's first and
+// takes the place the bit's rank gives; a vote that finds it set is a repeat
+// of the first vote's bin, or (rarely: 1,700 votes over 98,304 cells share
+// about 15) another bin of the same cell, which goes to a short list that is
+// sorted by itself and merged on the way out.  Two passes over the votes and
+// one over the bitmap, whatever the order the votes come in.
+// Bound: issue slots and latency together (half of each SM's threads, ~52%
+// issue; the per-thread cost of the bitmap pass is paid whatever the votes, so
+// small groups go with few votes).  500,000 reads of 100 bases on 3.1 Gbp
+// (1,700 votes a read): 14.9 -> 10.0 ms for the whole call; 500,000 of 150 on
+// 100 Mbp 3.77 -> 1.15, on 1 Mbp 3.01 -> 0.83; 200,000 on 800 Mbp, cap 100,
+// 3.27 -> 2.03.  What it replaced wrote every vote to memory, read it back and
+// sorted it by buckets with 256 threads a read; the same buckets sorted by
+// insertion here, without the trip through memory, took 17.5 ms.
+constexpr int kFastSeeds = 64;    // seeds per read
+constexpr int kStoredSeeds = 16;  // of which seed_lookup_kernel leaves the location ranges of the first
+constexpr int kFastExtra = 128;   // bins beside the first of their cell
+constexpr int kFastLoads = 4;     // locations in flight per thread
+constexpr int kFastHist = 64;     // the cap's vote threshold lies below this
+
+// T threads per read, each holding up to V votes in registers; CAP: reads may
+// have more bins than the cap keeps.
+template <int T, int V, bool CAP>
+struct FastGeo {
+    static_assert(V % 8 == 0 && V <= 32, "whole 16-byte groups of ranks, one bit per vote");
+    static constexpr int kVotes = V * T;
+    static constexpr int kWords = V * T;             // bitmap words: V per thread
+    static constexpr int kGroups = T == 32 ? 4 : 1;  // reads side by side in a CTA
+    // CTAs an SM should hold (registers): as many as the shared memory allows
+    static constexpr int kMinCtas = T == 32 ? 8 : T == 512 ? (V <= 16 ? 2 : 1) : (V <= 16 ? 1280 : 896) / T;
+};
+
+template <int T, int V, bool CAP>
+struct alignas(16) FastSmem {
+    using F = FastGeo<T, V, CAP>;
+    uint32_t map[F::kWords];                // (with a cap: then every bin, in order)
+    // the first vote's bin of every set cell, in order; from the back: the
+    // votes that found their bit set
+    uint32_t bin[F::kVotes];
+    uint16_t rank[F::kWords];               // set cells before each bitmap word (then every bin's votes)
+    uint32_t votes2[CAP ? F::kVotes / 2 : 4];  // with a cap: votes of bin[], two 16-bit counts a word
+    uint32_t extra[kFastExtra];             // as found, then without repeats
+    uint32_t sorted[kFastExtra];
+    uint32_t extra_votes[CAP ? kFastExtra : 1];
+    uint32_t hist[CAP ? kFastHist : 1];     // bins by votes (the last: and more)
+    uint32_t seed_at[kFastSeeds];           // vote i of the seed lies at seed_at + i
+    uint32_t seed_end[kFastSeeds];          // votes up to and with this seed
+    uint32_t warp_sum[32];
+    uint32_t n_set, n_extra, n_sorted;
+};
+
+// The seeds of each read of the batch, 16 lanes per read: (at, end) with vote
+// i < end of the seed at location at + i, as FastSmem holds them.  Done here,
+// a read's group starts its loads of locations two dependent loads after its
+// offsets instead of four (reads with more seeds look theirs up themselves).
+__global__ void seed_lookup_kernel(const uint32_t* __restrict__ idx_off, int k, const uint8_t* __restrict__ reads,
+                                   const int64_t* __restrict__ read_offsets, int64_t n, uint2* __restrict__ seeds) {
+    const int lane = threadIdx.x & 15;
+    const int64_t groups = (int64_t)gridDim.x * (blockDim.x >> 4);
+    const int64_t first = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+    const int64_t rounds = (n + groups - 1) / groups;
+    for (int64_t i = 0; i < rounds; i++) {  // the same for both halves of a warp
+        const int64_t r = first + i * groups;
+        int64_t ns = 0, ro = 0;
+        if (r < n) {
+            ro = read_offsets[r];
+            ns = n_seeds_of(read_offsets[r + 1] - ro, k);
+        }
+        uint32_t at = 0, m = 0, key;
+        if (ns <= kStoredSeeds && lane < ns && seed_key(reads + ro + (int64_t)lane * k, k, &key)) {
+            at = idx_off[key];
+            m = idx_off[key + 1] - at;
+        }
+        uint32_t x = m;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, x, o, 16);
+            if (lane >= o) x += y;
+        }
+        if (r < n) seeds[r * kStoredSeeds + lane] = make_uint2(at - (x - m), x);
+    }
+}
+
+template <int T>
+__device__ __forceinline__ void group_sync() {
+    if constexpr (T == 32) __syncwarp();
+    else __syncthreads();
+}
+
+// Exclusive prefix sum over the group's T threads; *total: the group's sum.
+template <int T>
+__device__ __forceinline__ uint32_t group_scan(uint32_t v, uint32_t* warp_sum, uint32_t* total) {
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x % T) >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += y;
+    }
+    if constexpr (T == 32) {
+        *total = __shfl_sync(kFull, x, 31);
+        return x - v;
+    } else {
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        uint32_t before = 0, sum = 0;
+#pragma unroll
+        for (int w = 0; w < T / 32; w++) {
+            const uint32_t y = warp_sum[w];
+            if (w < warp) before += y;
+            sum += y;
+        }
+        *total = sum;
+        __syncthreads();  // warp_sum may be used again
+        return before + x - v;
+    }
+}
+
+// Read r's kept bins (ascending) to H[hit_off[r] - h0 ...], their number to
+// kept[r]; false (nothing written) for a read this path cannot take.
+// cell_mul: floor(2^32 cells / n_bins), so that bin * cell_mul >> 32 spreads
+// the bin ids evenly and in order over the bitmap.  The whole group; ends
+// with the shared memory free for another read.
+template <int T, int V, bool CAP>
+__device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP>& sm, int64_t r, const uint32_t* __restrict__ idx_off,
+                                          const uint32_t* __restrict__ idx_pos, int k,
+                                          const uint8_t* __restrict__ reads,
+                                          const int64_t* __restrict__ read_offsets, const uint2* __restrict__ seeds,
+                                          const int64_t* __restrict__ hit_off, int64_t h0, FastDiv bin_div,
+                                          uint32_t last_bin, uint32_t cell_mul, int cap, uint32_t* __restrict__ H,
+                                          int64_t* __restrict__ kept) {
+    using F = FastGeo<T, V, CAP>;
+    const int t = threadIdx.x % T, lane = threadIdx.x & 31;
+    const int64_t base = hit_off[r] - h0, votes = hit_off[r + 1] - hit_off[r];
+    if (votes <= 0) {
+        if (t == 0) kept[r] = 0;
+        return true;
+    }
+    const int64_t ro = read_offsets[r];
+    const int64_t ns = n_seeds_of(read_offsets[r + 1] - ro, k);
+    if (votes > F::kVotes || ns > kFastSeeds) return false;
+    const int n = (int)votes;
+
+    // the seeds' location ranges (first warp), an empty bitmap
+#pragma unroll
+    for (int i = 0; i < F::kWords / 4 / T; i++)
+        reinterpret_cast<uint4*>(sm.map)[i * T + t] = make_uint4(0, 0, 0, 0);
+    if (ns <= kStoredSeeds) {
+        if (t < kStoredSeeds) {
+            const uint2 v = __ldg(seeds + r * kStoredSeeds + t);
+            sm.seed_at[t] = v.x;
+            sm.seed_end[t] = v.y;
+        }
+    } else if (t < 32) {
+        uint32_t before = 0;
+        for (int g = 0; g < (int)ns; g += 32) {
+            uint32_t at = 0, m = 0, key;
+            if (g + lane < ns && seed_key(reads + ro + (int64_t)(g + lane) * k, k, &key)) {
+                at = idx_off[key];
+                m = idx_off[key + 1] - at;
+            }
+            uint32_t x = m;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, x, o);
+                if (lane >= o) x += y;
+            }
+            sm.seed_at[g + lane] = at - (before + x - m);
+            sm.seed_end[g + lane] = before + x;
+            before += __shfl_sync(kFull, x, 31);
+        }
+    }
+    if (t == 0) sm.n_set = sm.n_extra = 0;
+    group_sync<T>();
+
+    // the votes' bins, in registers; a clear bit makes a vote its cell's first
+    uint32_t bin[V];
+    uint32_t is_first = 0;
+    int sd = 0;
+    uint32_t end = sm.seed_end[0], at = sm.seed_at[0];  // of seed sd
+#pragma unroll
+    for (int u0 = 0; u0 < V; u0 += kFastLoads) {
+        if (u0 * T >= n) break;  // the whole group
+        uint32_t off[kFastLoads];
+#pragma unroll
+        for (int u = 0; u < kFastLoads; u++) {
+            const int i = (u0 + u) * T + t;
+            if (i < n) {
+                while ((uint32_t)i >= end) {  // i < n = the last seed's end
+                    at = sm.seed_at[++sd];
+                    end = sm.seed_end[sd];
+                }
+                bin[u0 + u] = __ldg(idx_pos + (at + (uint32_t)i));
+                off[u] = (uint32_t)(sd * k);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kFastLoads; u++) {
+            const int i = (u0 + u) * T + t;
+            if (i < n) {
+                const uint32_t pos = bin[u0 + u];
+                uint32_t b = bin_div(pos > off[u] ? pos - off[u] : 0u);
+                b = b < last_bin ? b : last_bin;
+                bin[u0 + u] = b;
+                const uint32_t cell = __umulhi(b, cell_mul), m = 1u << (cell & 31);
+                if (!(atomicOr(&sm.map[cell >> 5], m) & m)) is_first |= 1u << (u0 + u);
+                else sm.bin[F::kVotes - 1 - atomicAdd(&sm.n_set, 1u)] = b;
+            }
+        }
+    }
+    group_sync<T>();
+
+    // set cells before each word: thread t owns words V t .. V t + V - 1
+    uint32_t n_first;
+    {
+        uint32_t c[V], sum = 0;
+#pragma unroll
+        for (int i = 0; i < V / 4; i++) {
+            const uint4 w = reinterpret_cast<const uint4*>(sm.map)[V / 4 * t + i];
+            c[4 * i] = __popc(w.x);
+            c[4 * i + 1] = __popc(w.y);
+            c[4 * i + 2] = __popc(w.z);
+            c[4 * i + 3] = __popc(w.w);
+        }
+#pragma unroll
+        for (int i = 0; i < V; i++) sum += c[i];
+        uint32_t o = group_scan<T>(sum, sm.warp_sum, &n_first);
+        uint4* dst = reinterpret_cast<uint4*>(sm.rank) + V / 8 * t;
+#pragma unroll
+        for (int g = 0; g < V / 8; g++) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                pk[i] = o | ((o + c[8 * g + 2 * i]) << 16);
+                o += c[8 * g + 2 * i] + c[8 * g + 2 * i + 1];
+            }
+            dst[g] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        }
+    }
+    group_sync<T>();
+    auto place = [&](uint32_t cell) {
+        return (uint32_t)sm.rank[cell >> 5] + __popc(sm.map[cell >> 5] & ((1u << (cell & 31)) - 1u));
+    };
+#pragma unroll
+    for (int u = 0; u < V; u++) {
+        if (u * T >= n) break;
+        if ((is_first >> u) & 1u) sm.bin[place(__umulhi(bin[u], cell_mul))] = bin[u];
+    }
+    group_sync<T>();
+    for (uint32_t i = t; i < sm.n_set; i += T) {
+        const uint32_t b = sm.bin[F::kVotes - 1 - i];
+        if (sm.bin[place(__umulhi(b, cell_mul))] != b) {
+            const uint32_t e = atomicAdd(&sm.n_extra, 1u);
+            if (e < kFastExtra) sm.extra[e] = b;
+        }
+    }
+    group_sync<T>();
+    const int n_extra = (int)sm.n_extra;
+    if (n_extra > kFastExtra) return false;
+    int n_sorted = 0;
+    if (n_extra > 0) {  // sort the extras, without repeats
+        constexpr uint32_t kNone = 0xFFFFFFFFu;  // no bin id
+        constexpr int kPer = (kFastExtra + T - 1) / T;
+        uint32_t x[kPer];
+        if (t == 0) sm.n_sorted = 0;
+#pragma unroll
+        for (int q = 0; q < kPer; q++) {
+            const int e = q * T + t;
+            x[q] = e < n_extra ? sm.extra[e] : kNone;
+            bool repeat = false;
+            if (e < n_extra)
+                for (int j = 0; j < e; j++) repeat |= sm.extra[j] == x[q];
+            if (repeat) x[q] = kNone;
+        }
+        group_sync<T>();
+#pragma unroll
+        for (int q = 0; q < kPer; q++) {
+            const int e = q * T + t;
+            if (e < n_extra) {
+                sm.extra[e] = x[q];
+                if (x[q] != kNone) atomicAdd(&sm.n_sorted, 1u);
+            }
+        }
+        group_sync<T>();
+#pragma unroll
+        for (int q = 0; q < kPer; q++) {
+            if (x[q] != kNone) {
+                int rank = 0;
+                for (int j = 0; j < n_extra; j++) rank += sm.extra[j] < x[q];
+                sm.sorted[rank] = x[q];
+            }
+        }
+        group_sync<T>();
+        n_sorted = (int)sm.n_sorted;
+    }
+    const uint32_t total = n_first + (uint32_t)n_sorted;
+    uint32_t* out = H + base;
+    auto extras_below = [&](uint32_t b) {
+        int lo = 0, hi = n_sorted;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (sm.sorted[mid] < b) lo = mid + 1;
+            else hi = mid;
+        }
+        return lo;
+    };
+    if (CAP && total > (uint32_t)cap) {
+        // the cap: the votes of every bin, the threshold v that leaves at
+        // least `cap` bins, then all bins above it and the first ones at it
+        for (int i = t; i < F::kVotes / 8; i += T)
+            reinterpret_cast<uint4*>(sm.votes2)[i] = make_uint4(0, 0, 0, 0);
+        for (int e = t; e < kFastExtra; e += T) sm.extra_votes[e] = 0;
+        for (int e = t; e < kFastHist; e += T) sm.hist[e] = 0;
+        group_sync<T>();
+#pragma unroll
+        for (int u = 0; u < V; u++) {
+            if (u * T >= n) break;
+            if (u * T + t < n) {
+                const uint32_t p = place(__umulhi(bin[u], cell_mul));
+                if (sm.bin[p] == bin[u]) atomicAdd(&sm.votes2[p >> 1], 1u << (16 * (p & 1)));
+                else atomicAdd(&sm.extra_votes[extras_below(bin[u])], 1u);
+            }
+        }
+        group_sync<T>();
+        auto votes_of = [&](uint32_t j) { return (sm.votes2[j >> 1] >> (16 * (j & 1))) & 0xFFFFu; };
+        uint32_t ones = 0;  // most bins: counted apart, without atomics on one word
+        for (uint32_t j = t; j < n_first; j += T) {
+            const uint32_t v = votes_of(j);
+            if (v == 1) ones++;
+            else atomicAdd(&sm.hist[v < kFastHist - 1 ? v : kFastHist - 1], 1u);
+        }
+        constexpr int kPerE = (kFastExtra + T - 1) / T;
+        uint32_t e_bin[kPerE], e_votes[kPerE], e_at[kPerE];
+#pragma unroll
+        for (int q = 0; q < kPerE; q++) {
+            const int e = q * T + t;
+            if (e < n_sorted) {
+                e_bin[q] = sm.sorted[e];
+                e_votes[q] = sm.extra_votes[e];
+                const uint32_t p = place(__umulhi(e_bin[q], cell_mul));
+                e_at[q] = p + (sm.bin[p] < e_bin[q]) + e;
+                atomicAdd(&sm.hist[e_votes[q] < kFastHist - 1 ? e_votes[q] : kFastHist - 1], 1u);
+            }
+        }
+        ones = __reduce_add_sync(kFull, ones);
+        if (lane == 0 && ones) atomicAdd(&sm.hist[1], ones);
+        group_sync<T>();  // the bitmap and the ranks are free
+        const uint32_t h0v = sm.hist[2 * lane], h1v = sm.hist[2 * lane + 1];
+        uint32_t ge = h0v + h1v;  // bins of at least 2 lane votes
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_down_sync(kFull, ge, o);
+            if (lane + o < 32) ge += y;
+        }
+        const uint32_t c32 = (uint32_t)cap;
+        const uint32_t v_lane = ge - h0v >= c32 ? 2 * lane + 1 : ge >= c32 ? 2 * lane : 0;
+        const uint32_t v_star = __reduce_max_sync(kFull, v_lane);
+        if (v_star == kFastHist - 1) return false;
+        // bins above the threshold: ge at v_star + 1
+        const uint32_t above_even = __shfl_sync(kFull, ge, ((v_star + 1) >> 1) & 31);
+        const uint32_t above_odd = __shfl_sync(kFull, ge - h0v, ((v_star + 1) >> 1) & 31);
+        const uint32_t need = c32 - ((v_star + 1) & 1 ? above_odd : above_even);
+        for (uint32_t j = t; j < n_first; j += T) {
+            const uint32_t b = sm.bin[j], to = j + extras_below(b);
+            sm.map[to] = b;
+            sm.rank[to] = (uint16_t)votes_of(j);
+        }
+#pragma unroll
+        for (int q = 0; q < kPerE; q++)
+            if (q * T + t < n_sorted) {
+                sm.map[e_at[q]] = e_bin[q];
+                sm.rank[e_at[q]] = (uint16_t)e_votes[q];
+            }
+        group_sync<T>();
+        uint32_t n_gt = 0, n_eq = 0;  // before this chunk of 4 T bins
+        for (uint32_t c0 = 0; c0 < total; c0 += 4 * T) {
+            uint32_t gt = 0, eq = 0;
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const uint32_t j = c0 + 4 * t + q;
+                const uint32_t v = j < total ? sm.rank[j] : 0u;
+                gt |= (uint32_t)(v > v_star) << q;
+                eq |= (uint32_t)(v == v_star) << q;  // v_star >= 1
+            }
+            uint32_t both;
+            const uint32_t o =
+                group_scan<T>((uint32_t)__popc(gt) | ((uint32_t)__popc(eq) << 16), sm.warp_sum, &both);
+            uint32_t g = n_gt + (o & 0xFFFFu), q_eq = n_eq + (o >> 16);
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if ((gt >> q) & 1u) {
+                    out[g + (q_eq < need ? q_eq : need)] = sm.map[c0 + 4 * t + q];
+                    g++;
+                } else if ((eq >> q) & 1u) {
+                    if (q_eq < need) out[g + q_eq] = sm.map[c0 + 4 * t + q];
+                    q_eq++;
+                }
+            }
+            n_gt += both & 0xFFFFu;
+            n_eq += both >> 16;
+        }
+        if (t == 0) kept[r] = cap;
+        return true;
+    }
+
+    // extra e goes in before first vote number cut_e (its bin's rank among
+    // them): a warp's 32 consecutive first votes are mostly between two cuts
+    constexpr int kPerCut = kFastExtra / 32;
+    uint32_t cut[kPerCut];  // of extras 32 q + lane, in every warp
+    const int cuts = (n_sorted + 31) >> 5;
+#pragma unroll
+    for (int q = 0; q < kPerCut; q++) {
+        cut[q] = 0xFFFFFFFFu;
+        const int e = 32 * q + lane;
+        if (q < cuts && e < n_sorted) {
+            const uint32_t b = sm.sorted[e];
+            const uint32_t p = place(__umulhi(b, cell_mul));  // its cell's first vote
+            cut[q] = p + (sm.bin[p] < b);
+            if (t < 32) out[cut[q] + e] = b;
+        }
+    }
+    for (uint32_t j0 = t - lane; j0 < n_first; j0 += T) {
+        const uint32_t j = j0 + lane;
+        uint32_t shift = 0;
+        bool split = false;
+#pragma unroll
+        for (int q = 0; q < kPerCut; q++)
+            if (q < cuts) {
+                shift += __popc(__ballot_sync(kFull, cut[q] <= j0));
+                split |= __ballot_sync(kFull, cut[q] > j0 && cut[q] <= j0 + 31) != 0;
+            }
+        if (j < n_first) {
+            const uint32_t b = sm.bin[j];
+            out[j + (split ? (uint32_t)extras_below(b) : shift)] = b;
+        }
+    }
+    if (t == 0) kept[r] = total;
+    return true;
+}
+
+// Every read of the batch (list == null) or the listed ones, a group of T
+// threads each; those that fast_read does not take are appended to
+// slow[0 .. *n_slow).
+template <int T, int V, bool CAP>
+__global__ void __launch_bounds__(T * FastGeo<T, V, CAP>::kGroups, FastGeo<T, V, CAP>::kMinCtas)
+seed_fast_kernel(const uint32_t* __restrict__ idx_off, const uint32_t* __restrict__ idx_pos, int k,
+                 const uint8_t* __restrict__ reads, const int64_t* __restrict__ read_offsets,
+                 const uint2* __restrict__ seeds, int64_t n_reads, const uint32_t* __restrict__ list,
+                 const uint32_t* __restrict__ n_list, const int64_t* __restrict__ hit_off, int64_t h0,
+                 FastDiv bin_div, uint32_t last_bin,
+                 uint32_t cell_mul, int cap, uint32_t* __restrict__ H, int64_t* __restrict__ kept,
+                 uint32_t* __restrict__ slow, uint32_t* __restrict__ n_slow) {
+    using F = FastGeo<T, V, CAP>;
+    extern __shared__ __align__(16) uint8_t fast_smem_raw[];
+    const int group = threadIdx.x / T;
+    FastSmem<T, V, CAP>& sm = reinterpret_cast<FastSmem<T, V, CAP>*>(fast_smem_raw)[group];
+    const int64_t n = list ? (int64_t)*n_list : n_reads;
+    for (int64_t i = (int64_t)blockIdx.x * F::kGroups + group; i < n; i += (int64_t)gridDim.x * F::kGroups) {
+        const int64_t r = list ? (int64_t)list[i] : i;
+        const bool taken = fast_read<T, V, CAP>(sm, r, idx_off, idx_pos, k, reads, read_offsets, seeds, hit_off, h0,
+                                        bin_div, last_bin, cell_mul, cap, H, kept);
+        if (!taken && threadIdx.x % T == 0) slow[atomicAdd(n_slow, 1u)] = (uint32_t)r;
+        group_sync<T>();
+    }
+}
+
+// The votes of the listed reads list[0 .. *n_list) of the batch: read r's
+// bins at H[hit_off[r] - h0 ...], one CTA per read, its warps taking the seeds
+// in turn (a listed read has thousands of locations per seed).
 __global__ void seed_expand_kernel(const uint32_t* __restrict__ idx_off, const uint32_t* __restrict__ idx_pos, int k,
                                    const uint8_t* __restrict__ reads, const int64_t* __restrict__ read_offsets,
-                                   int64_t n, const int64_t* __restrict__ hit_off, int64_t h0, uint32_t bin_len,
+                                   const uint32_t* __restrict__ list, const uint32_t* __restrict__ n_list,
+                                   const int64_t* __restrict__ hit_off, int64_t h0, uint32_t bin_len,
                                    uint32_t last_bin, uint32_t* __restrict__ H) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int64_t n = *n_list;
+    for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
+        const int64_t r = list[i];
         const int64_t ro = read_offsets[r], L = read_offsets[r + 1] - ro;
         const int64_t ns = n_seeds_of(L, k);
-        int64_t w = hit_off[r] - h0;
+        int64_t w = hit_off[r] - h0;  // first vote of this group of 32 seeds
         for (int64_t g = 0; g < ns; g += 32) {
-            // lane sd of this group looks up seed g + sd
-            uint32_t a = 0, b = 0;
-            if (g + lane < ns) {
-                uint32_t key;
-                if (seed_key(reads + ro + (g + lane) * k, k, &key)) {
-                    a = idx_off[key];
-                    b = idx_off[key + 1];
-                }
+            // lane sd of every warp looks up seed g + sd
+            uint32_t a = 0, m = 0, key;
+            if (g + lane < ns && seed_key(reads + ro + (g + lane) * k, k, &key)) {
+                a = idx_off[key];
+                m = idx_off[key + 1] - a;
             }
-            const int m = ns - g < 32 ? (int)(ns - g) : 32;
-            for (int sd = 0; sd < m; sd++) {
-                const uint32_t sa = __shfl_sync(kFull, a, sd), sb = __shfl_sync(kFull, b, sd);
+            int64_t x = m;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t y = __shfl_up_sync(kFull, x, o);
+                if (lane >= o) x += y;
+            }
+            const int cnt = ns - g < 32 ? (int)(ns - g) : 32;
+            for (int sd = warp; sd < cnt; sd += warps) {
+                const uint32_t sa = __shfl_sync(kFull, a, sd), sm = __shfl_sync(kFull, m, sd);
+                const int64_t to = w + __shfl_sync(kFull, x, sd) - sm;
                 const uint32_t o = (uint32_t)((g + sd) * k);
-                for (uint32_t j = sa + lane; j < sb; j += 32) {
-                    const uint32_t p = __ldg(idx_pos + j);
+                for (uint32_t j = lane; j < sm; j += 32) {
+                    const uint32_t p = __ldg(idx_pos + sa + j);
                     const uint32_t start = p > o ? p - o : 0u;
                     const uint32_t bin = start / bin_len;
-                    H[w + (j - sa)] = bin < last_bin ? bin : last_bin;
+                    H[to + j] = bin < last_bin ? bin : last_bin;
                 }
-                w += sb - sa;
             }
+            w += __shfl_sync(kFull, x, 31);
         }
     }
 }
@@ -498,49 +994,98 @@ __device__ __forceinline__ int64_t dedupe_read(uint32_t* A, uint32_t* B, I n, in
     return n_keep;
 }
 
-// One CTA per read of the batch: its votes sorted, runs found, the cap
-// applied and the kept bins (ascending) written to H[hit_off[r] - h0 ...],
-// their number to kept[r].  Reads of up to kDedupSmem votes work in shared
-// memory (bucket sort, else radix sort; run starts in the sort's second
-// buffer).  Longer reads use S, scratch of 8 bytes per vote, as 2n u32: run
-// starts from the front, the back half as the radix sort's second buffer,
-// then their list after the starts before it is copied to H.  `passes`:
-// radix digits covering every bin id (even); `bits`: bits of the largest bin id.
+// The listed reads list[0 .. *n_list) of the batch, one CTA at a time: votes
+// sorted, runs found, the cap applied and the kept bins (ascending) written to
+// H[hit_off[r] - h0 ...], their number to kept[r].  Reads of up to kDedupSmem
+// votes work in shared memory (bucket sort, else radix sort; run starts in the
+// sort's second buffer).  Longer reads use S, scratch of 8 bytes per vote, as
+// 2n u32: run starts from the front, the back half as the radix sort's second
+// buffer, then their list after the starts before it is copied to H.
+// `passes`: radix digits covering every bin id (even); `bits`: bits of the
+// largest bin id.
 __global__ void __launch_bounds__(kDedupThreads)
-seed_dedupe_kernel(const int64_t* __restrict__ hit_off, int64_t h0, int cap, int passes, int bits,
+seed_dedupe_kernel(const uint32_t* __restrict__ read_list, const uint32_t* __restrict__ n_list,
+                   const int64_t* __restrict__ hit_off, int64_t h0, int cap, int passes, int bits,
                    uint32_t* __restrict__ H,
                    unsigned long long* __restrict__ S, int64_t* __restrict__ kept) {
     extern __shared__ uint32_t dedupe_smem[];
     __shared__ int64_t ws[32];
     __shared__ uint32_t ws32[32];
     __shared__ unsigned int max_votes;
-    const int64_t r = blockIdx.x;
-    const int64_t base = hit_off[r] - h0, n = hit_off[r + 1] - hit_off[r];
-    if (n <= 0) {
-        if (threadIdx.x == 0) kept[r] = 0;
-        return;
+    const uint32_t n_reads = *n_list;
+    for (uint32_t i_list = blockIdx.x; i_list < n_reads; i_list += gridDim.x) {
+        const int64_t r = read_list[i_list];
+        const int64_t base = hit_off[r] - h0, n = hit_off[r + 1] - hit_off[r];  // n > 0
+        uint32_t* st = reinterpret_cast<uint32_t*>(S + base);  // 2n u32 of scratch
+        int64_t n_keep;
+        if (n <= kDedupSmem) {
+            uint32_t* A_s = dedupe_smem;
+            uint32_t* B_s = dedupe_smem + kDedupPadded;
+            uint32_t* cnt = dedupe_smem + 2 * kDedupPadded;
+            const int ni = (int)n;
+            for (int i = threadIdx.x; i < ni; i += blockDim.x) A_s[rx_at<true>(i)] = H[base + i];
+            __syncthreads();
+            // the run starts go to B_s, free once A_s is sorted
+            n_keep = dedupe_read<true, int>(A_s, B_s, ni, cap, passes, bits, cnt, B_s, H + base, ws32, ws,
+                                            &max_votes);
+        } else {
+            uint32_t* cnt = dedupe_smem + 2 * kDedupPadded;
+            // the list is built after the starts (st + n: the sort's buffer, free by then)
+            uint32_t* list = st + n;
+            n_keep = dedupe_read<false, int64_t>(H + base, st + n, n, cap, passes, bits, cnt, st, list, ws32, ws,
+                                                 &max_votes);
+            __syncthreads();
+            for (int64_t j = threadIdx.x; j < n_keep; j += blockDim.x) H[base + j] = list[j];
+        }
+        if (threadIdx.x == 0) kept[r] = n_keep;
+        __syncthreads();  // the shared arrays are free for the next read
     }
-    uint32_t* st = reinterpret_cast<uint32_t*>(S + base);  // 2n u32 of scratch
-    int64_t n_keep;
-    if (n <= kDedupSmem) {
-        uint32_t* A_s = dedupe_smem;
-        uint32_t* B_s = dedupe_smem + kDedupPadded;
-        uint32_t* cnt = dedupe_smem + 2 * kDedupPadded;
-        const int ni = (int)n;
-        for (int i = threadIdx.x; i < ni; i += blockDim.x) A_s[rx_at<true>(i)] = H[base + i];
-        __syncthreads();
-        // the run starts go to B_s, free once A_s is sorted
-        n_keep = dedupe_read<true, int>(A_s, B_s, ni, cap, passes, bits, cnt, B_s, H + base, ws32, ws, &max_votes);
-    } else {
-        uint32_t* cnt = dedupe_smem + 2 * kDedupPadded;
-        // the list is built after the starts (st + n: the sort's buffer, free by then)
-        uint32_t* list = st + n;
-        n_keep = dedupe_read<false, int64_t>(H + base, st + n, n, cap, passes, bits, cnt, st, list, ws32, ws,
-                                             &max_votes);
-        __syncthreads();
-        for (int64_t j = threadIdx.x; j < n_keep; j += blockDim.x) H[base + j] = list[j];
+}
+
+struct FastArgs {
+    const grim_seed_index* idx;
+    const uint8_t* reads;
+    const int64_t* read_offsets;
+    const uint2* seeds;
+    int64_t nb;
+    const int64_t* hit_off;
+    int64_t h0;
+    int bin_len;
+    int64_t n_bins;
+    int cap;
+    uint32_t* H;
+    int64_t* kept;
+};
+
+template <int T, int V, bool CAP>
+cudaError_t launch_fast(const FastArgs& a, const uint32_t* list, const uint32_t* n_list, uint32_t* slow,
+                        uint32_t* n_slow, cudaStream_t s) {
+    using F = FastGeo<T, V, CAP>;
+    constexpr size_t smem = sizeof(FastSmem<T, V, CAP>) * F::kGroups;
+    static DeviceCache attr[64];  // per device
+    const int dev = a.idx->device;
+    if (smem > 48 * 1024 && dev >= 0 && dev < 64 && !attr[dev].load()) {
+        const cudaError_t e = cudaFuncSetAttribute(seed_fast_kernel<T, V, CAP>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr[dev].store(1);
     }
-    if (threadIdx.x == 0) kept[r] = n_keep;
+    const uint64_t mul = ((uint64_t)(32 * F::kWords) << 32) / (uint64_t)a.n_bins;
+    int64_t blocks = (a.nb + F::kGroups - 1) / F::kGroups;
+    if (list && blocks > 4 * sm_count()) blocks = 4 * sm_count();  // few, taken in turn
+    seed_fast_kernel<T, V, CAP><<<grim::fault_grid((unsigned)blocks), T * F::kGroups, smem, s>>>(
+        a.idx->offsets, a.idx->positions, a.idx->k, a.reads, a.read_offsets, a.seeds, a.nb, list, n_list, a.hit_off, a.h0,
+        FastDiv((uint32_t)a.bin_len), (uint32_t)(a.n_bins - 1),
+        (uint32_t)(mul < 0xFFFFFFFFull ? mul : 0xFFFFFFFFull), a.cap, a.H, a.kept, slow, n_slow);
+    return cudaGetLastError();
+}
+
+// A cap that no read the kernel takes can exceed needs no votes per bin.
+template <int T, int V>
+cudaError_t launch_seed_fast(const FastArgs& a, const uint32_t* list, const uint32_t* n_list, uint32_t* slow,
+                             uint32_t* n_slow, cudaStream_t s) {
+    return a.cap >= FastGeo<T, V, true>::kVotes ? launch_fast<T, V, false>(a, list, n_list, slow, n_slow, s)
+                                                : launch_fast<T, V, true>(a, list, n_list, slow, n_slow, s);
 }
 
 // cand_bins[cand_off[r] ...] <- the kept bins of read r (warp per read),
@@ -553,8 +1098,16 @@ __global__ void seed_copy_kernel(const uint32_t* __restrict__ H, const int64_t* 
     for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
         const uint32_t* src = H + (hit_off[r] - h0);
         const int64_t d = cand_off[r], m = cand_off[r + 1] - d;
-        for (int64_t j = lane; j < m; j += 32)
-            if (d + j < capacity) cand_bins[d + j] = src[j];
+        const int64_t room = capacity - d < m ? capacity - d : m;
+        int64_t j = lane;
+        for (; j + 7 * 32 < room; j += 8 * 32) {  // eight loads in flight per lane
+            uint32_t v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) v[u] = src[j + 32 * u];
+#pragma unroll
+            for (int u = 0; u < 8; u++) cand_bins[d + j + 32 * u] = v[u];
+        }
+        for (; j < room; j += 32) cand_bins[d + j] = src[j];
     }
 }
 
@@ -824,10 +1377,15 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
     uint32_t* H = nullptr;
     unsigned long long* S = nullptr;
     int64_t* kept = nullptr;
+    uint2* seeds = nullptr;    // location ranges of the batch's seeds
+    uint32_t* slow = nullptr;  // lists of the reads the fast path leaves
     int64_t cap_votes = 0;
     if (e == cudaSuccess && rc == GRIM_OK) {
         const int64_t max_nb = n_reads < kMaxReads ? n_reads : kMaxReads;
         e = grim::scratch_alloc((void**)&kept, (size_t)max_nb * 8, s);
+        if (e == cudaSuccess)
+            e = grim::scratch_alloc((void**)&seeds, (size_t)max_nb * grim::kStoredSeeds * sizeof(uint2), s);
+        if (e == cudaSuccess) e = grim::scratch_alloc((void**)&slow, (size_t)(3 * max_nb + 4) * 4, s);
         if (e == cudaSuccess) {
             grim::set_value_kernel<int64_t><<<grim::fault_grid(1), 1, 0, s>>>(cand_offsets, 0, nullptr);
             e = cudaGetLastError();
@@ -855,12 +1413,36 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         }
         const int64_t wb = (nb * 32 + threads - 1) / threads;
         const unsigned bb = (unsigned)(wb < 65535 ? wb : 65535);
-        if (votes > 0)
-            grim::seed_expand_kernel<<<grim::fault_grid(bb), threads, 0, s>>>(
-                    idx->offsets, idx->positions, idx->k, reads, read_offsets + r0, nb, hit_off + r0, h0,
-                    (uint32_t)bin_len, (uint32_t)(n_bins - 1), H);
-        grim::seed_dedupe_kernel<<<grim::fault_grid((unsigned)nb), grim::kDedupThreads, grim::kDedupSmemBytes, s>>>(
-            hit_off + r0, h0, cap, passes, bits, H, S, kept);
+        // three lists and their lengths: reads of more votes than the batch's
+        // group size takes (tried again with larger groups), and the rest
+        uint32_t *n_list = slow, *list0 = slow + 4, *list1 = list0 + nb, *list2 = list1 + nb;
+        e = cudaMemsetAsync(n_list, 0, 16, s);
+        if (e != cudaSuccess) break;
+        // threads per read by the batch's mean votes, with room for about three
+        // times it (at 1,700 votes: 256 x 16 10.0 ms a call, 128 x 24 11.1,
+        // whose reads of over 3,072 votes then take the larger groups)
+        const int64_t mean = votes / nb;
+        const int64_t lookup_blocks = (nb * 16 + threads - 1) / threads;
+        grim::seed_lookup_kernel<<<grim::fault_grid((unsigned)(lookup_blocks < 65535 ? lookup_blocks : 65535)),
+                                   threads, 0, s>>>(idx->offsets, idx->k, reads, read_offsets + r0, nb, seeds);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) break;
+        const grim::FastArgs fa{idx,     reads,  read_offsets + r0, seeds, nb,  hit_off + r0, h0,
+                                bin_len, n_bins, cap,               H,     kept};
+        if (mean <= 160) e = grim::launch_seed_fast<32, 16>(fa, nullptr, nullptr, list0, n_list, s);
+        else if (mean <= 400) e = grim::launch_seed_fast<64, 16>(fa, nullptr, nullptr, list0, n_list, s);
+        else if (mean <= 800) e = grim::launch_seed_fast<64, 24>(fa, nullptr, nullptr, list0, n_list, s);
+        else if (mean <= 1200) e = grim::launch_seed_fast<128, 24>(fa, nullptr, nullptr, list0, n_list, s);
+        else e = grim::launch_seed_fast<256, 16>(fa, nullptr, nullptr, list0, n_list, s);
+        if (e == cudaSuccess) e = grim::launch_seed_fast<256, 24>(fa, list0, n_list, list1, n_list + 1, s);
+        if (e == cudaSuccess) e = grim::launch_seed_fast<512, 24>(fa, list1, n_list + 1, list2, n_list + 2, s);
+        if (e != cudaSuccess) break;
+        const unsigned few = (unsigned)(nb < 4 * grim::sm_count() ? nb : 4 * grim::sm_count());
+        grim::seed_expand_kernel<<<grim::fault_grid(few), threads, 0, s>>>(
+                idx->offsets, idx->positions, idx->k, reads, read_offsets + r0, list2, n_list + 2, hit_off + r0, h0,
+                (uint32_t)bin_len, (uint32_t)(n_bins - 1), H);
+        grim::seed_dedupe_kernel<<<grim::fault_grid(few), grim::kDedupThreads, grim::kDedupSmemBytes, s>>>(
+            list2, n_list + 2, hit_off + r0, h0, cap, passes, bits, H, S, kept);
         e = cudaGetLastError();
         // offsets continue from the previous batch's total in cand_offsets[r0]
         if (e == cudaSuccess) rc = grim::exclusive_scan<int64_t>(kept, cand_offsets + r0, nb, 0, s, cand_offsets + r0);
@@ -877,6 +1459,8 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
     if (H) cudaFreeAsync(H, s);
     if (S) cudaFreeAsync(S, s);
     if (kept) cudaFreeAsync(kept, s);
+    if (slow) cudaFreeAsync(slow, s);
+    if (seeds) cudaFreeAsync(seeds, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFreeAsync(hit_off, s);
     cudaFreeAsync(info, s);
