@@ -69,41 +69,70 @@ __device__ __forceinline__ void csa(uint32_t& hi, uint32_t& lo, uint32_t a, uint
     lo = u ^ c;
 }
 
-// popcount(x AND p0) + 2 popcount(x AND p1) over a lane's 8 words (two
-// 16-byte vectors), p1 only when NP == 2.  Full adders first reduce words
-// of equal weight (Harley-Seal), so 6 popcounts (4 for one plane) replace
-// 16 (8): for rows of 512 bytes the popcount pipe's latency, not issue
-// slots, limits the gather.
-template <int NP>
-__device__ __forceinline__ uint32_t row_sum_csa(const uint4 (&v)[2], const uint4 (&p)[NP][2]) {
+// A lane's weighted count of one row slice: sum_p 2^p popcount(x AND plane_p)
+// over its 8 words x (two 16-byte vectors), for reads of NP count planes.
+//
+// POPC runs at 16 lanes a clock and SM, a quarter of the logic rate, so
+// counting every ANDed word by itself is bound by that pipe (q = 5 with two
+// planes: 16 POPC = 128 cycles of a scheduler per warp step against 48 of
+// logic).  Two things take POPCs out:
+//  - full adders over words of equal weight (Harley-Seal): 2 three-input
+//    logic ops in place of one POPC and its add;
+//  - the top plane of a read is nearly empty (150 bases, q = 5: ~9 of 1,024
+//    tokens occur twice).  When no two of the four words of a vector share
+//    a bit in it (`kSparse`, checked once per read by sparse_plane), their
+//    ANDed words are simply ORed together - one three-input op per word -
+//    and counted once per vector.
+// kSparse: the top plane NP - 1 >= 1 is folded that way.
+// 1M reads of 150 bases, 75 candidates each, bank in L2: 1.55 -> 1.49 ms;
+// 200,000 reads of 1,000 candidates 3.20 -> 2.78; q = 6, 290M checks, 18.2 ->
+// 16.6 (there the bank is read from HBM, and the adders were in use before).
+template <int NP, bool kSparse>
+__device__ __forceinline__ uint32_t row_sum8(const uint4 (&v)[2], const uint4 (&p)[NP][2]) {
+    uint32_t sum = 0;
+    if constexpr (kSparse) {
+        const uint4(&t)[2] = p[NP - 1];
+        uint32_t o0 = v[0].x & t[0].x, o1 = v[1].x & t[1].x;
+        o0 |= v[0].y & t[0].y;
+        o1 |= v[1].y & t[1].y;
+        o0 |= v[0].z & t[0].z;
+        o1 |= v[1].z & t[1].z;
+        o0 |= v[0].w & t[0].w;
+        o1 |= v[1].w & t[1].w;
+        sum = (__popc(o0) + __popc(o1)) << (NP - 1);
+    }
     const uint32_t a0 = v[0].x & p[0][0].x, a1 = v[0].y & p[0][0].y, a2 = v[0].z & p[0][0].z,
                    a3 = v[0].w & p[0][0].w, a4 = v[1].x & p[0][1].x, a5 = v[1].y & p[0][1].y,
                    a6 = v[1].z & p[0][1].z, a7 = v[1].w & p[0][1].w;
-    uint32_t c1, s1, c2, s2, c3, s3;
+    uint32_t c1, s1, c2, s2, c3, s3, d1, s4;
     csa(c1, s1, a0, a1, a2);
     csa(c2, s2, a3, a4, a5);
     csa(c3, s3, s1, s2, a6);
-    if constexpr (NP == 1) {
-        uint32_t d1, s4;
-        csa(d1, s4, c1, c2, c3);
-        return __popc(s3) + __popc(a7) + 2 * __popc(s4) + 4 * __popc(d1);
+    csa(d1, s4, c1, c2, c3);
+    sum += __popc(s3) + __popc(a7);
+    if constexpr (NP - (kSparse ? 1 : 0) == 1) {
+        return sum + 2 * __popc(s4) + 4 * __popc(d1);
     } else {
+        static_assert(NP - (kSparse ? 1 : 0) == 2, "two dense planes at most");
         const uint32_t b0 = v[0].x & p[1][0].x, b1 = v[0].y & p[1][0].y, b2 = v[0].z & p[1][0].z,
                        b3 = v[0].w & p[1][0].w, b4 = v[1].x & p[1][1].x, b5 = v[1].y & p[1][1].y,
                        b6 = v[1].z & p[1][1].z, b7 = v[1].w & p[1][1].w;
-        // weight 2: c1 c2 c3 b0..b7
-        uint32_t d1, s4, d2, s5, d3, s6, d4, s7, d5, s8;
-        csa(d1, s4, c1, c2, c3);
+        uint32_t d2, s5, d3, s6, d4, s7;  // weight 2: s4 b0..b7
         csa(d2, s5, b0, b1, b2);
         csa(d3, s6, b3, b4, b5);
         csa(d4, s7, s4, s5, s6);
-        csa(d5, s8, s7, b6, b7);
-        // weight 4: d1..d5
-        uint32_t e1, s9, e2, s10;
-        csa(e1, s9, d1, d2, d3);
-        csa(e2, s10, s9, d4, d5);
-        return __popc(s3) + __popc(a7) + 2 * __popc(s8) + 4 * __popc(s10) + 8 * (__popc(e1) + __popc(e2));
+        return sum + 2 * (__popc(s7) + __popc(b6) + __popc(b7)) +
+               4 * (__popc(d1) + __popc(d2) + __popc(d3) + __popc(d4));
     }
+}
+
+// Whether no two words of each of the lane's vectors share a bit, over the
+// whole warp (see row_sum8).  `t`: the lane's two vectors of the plane.
+__device__ __forceinline__ bool sparse_plane(const uint4& t0, const uint4& t1) {
+    auto shared_bits = [](const uint4& m) {
+        return (m.x & m.y) | ((m.x | m.y) & m.z) | ((m.x | m.y | m.z) & m.w);
+    };
+    return !__any_sync(kFull, (shared_bits(t0) | shared_bits(t1)) != 0);
 }
 
 // The candidate stream of one read.  Step k scores rows k*BPS .. k*BPS+BPS-1
@@ -230,10 +259,10 @@ struct StepReducer {
     }
 };
 
-// Score the read's candidates.  NP > 0: NP planes held in registers;
-// NP == 0: P planes read from shared memory.  cands / pass / sums point at
-// the read's first candidate.
-template <int Q, int NP, bool DEEP>
+// Score the read's candidates.  NP > 0: NP planes held in registers (SPARSE:
+// the top one folded, see row_sum8); NP == 0: P planes read from shared
+// memory.  cands / pass / sums point at the read's first candidate.
+template <int Q, int NP, bool DEEP, bool SPARSE = false>
 __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __restrict__ planes, int P, int T,
                                            int n, const uint32_t* __restrict__ cands,
                                            const uint32_t* __restrict__ bank, uint32_t n_bins32,
@@ -282,8 +311,8 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
                 }
                 // score this step's rows
                 const uint4 (&v)[G::kVPL] = st.r[tl % S::kBufs];
-                if constexpr (NP > 0 && NP <= 2 && Q >= 6 && G::kVPL == 2) {
-                    part = row_sum_csa<NP>(v, pl);
+                if constexpr (NP > 0 && G::kVPL == 2) {
+                    part = row_sum8<NP, SPARSE>(v, pl);
                 } else if (NP > 0) {
 #pragma unroll
                     for (int p = 0; p < (NP > 0 ? NP : 1); p++) {
@@ -381,17 +410,21 @@ __device__ __forceinline__ int planes_from_counters(uint32_t* __restrict__ plane
     return used;
 }
 
-// Shared-memory set-up of a gather CTA: zeroed count planes.
+// First word of a warp's plane area that must be zero between reads: its
+// upper half for q <= 5 (the byte counters; the planes proper are written
+// whole), all of it for q = 6 (planes only ever built by carries).
 template <int Q>
-__device__ __forceinline__ void gather_cta_setup(uint4* smem, int warps) {
-    using G = GatherGeo<Q>;
-    uint32_t* planes_all = reinterpret_cast<uint32_t*>(smem);
-    for (int i = threadIdx.x; i < warps * G::kPlaneWords; i += blockDim.x) planes_all[i] = 0;
-    __syncthreads();
+constexpr int kCleanFrom = Q <= 5 ? 8 * GatherGeo<Q>::kRowWords : 0;
+
+// Shared-memory set-up of a gather warp.
+template <int Q>
+__device__ __forceinline__ void gather_warp_setup(uint32_t* planes, int lane) {
+    for (int i = kCleanFrom<Q> + lane; i < GatherGeo<Q>::kPlaneWords; i += 32) planes[i] = 0;
+    __syncwarp();
 }
 
 // The whole filter for read r, by one warp (steps 0-5 above).  The warp's
-// count planes are zero on entry and left zero on exit.
+// plane area is zero from kCleanFrom on at entry, and left so.
 // ro, re: the read's bases; co, ce: its candidates; e: its edit budget.
 template <int Q, bool DEEP>
 __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, int64_t ce, int e,
@@ -400,7 +433,8 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
                                             const uint32_t* __restrict__ cand_bins, uint8_t* __restrict__ pass,
                                             uint16_t* __restrict__ sums, uint32_t* __restrict__ planes, int lane,
                                             uint32_t& flags) {
-    constexpr int RW = GatherGeo<Q>::kRowWords;
+    using G = GatherGeo<Q>;
+    constexpr int RW = G::kRowWords;
     const uint4* planes4 = reinterpret_cast<const uint4*>(planes);
     if (ce < co) {  // nothing sensible to write for this read
         flags |= GRIM_FLAG_BAD_OFFSETS;
@@ -438,6 +472,8 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
         __syncwarp();
         used = planes_from_counters<Q>(planes, lane);
     } else {  // q = 6 and longer reads: a carry chain of atomicXor per token
+        for (int i = lane; i < kCleanFrom<Q>; i += 32) planes[i] = 0;
+        __syncwarp();
         int top = -1;  // highest plane this lane set
         for_each_token5<Q>(rd, L, lane, bad_base, [&](uint32_t tok) {
             const uint32_t w = tok >> 5, m = 1u << (tok & 31);
@@ -462,24 +498,36 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
     if (co < ce) {
         if (bad_read || used == 0)
             write_constant(co, ce, cand_bins, n_bins, !bad_read && T <= 0, pass, sums, lane, flags);
-        else if (used == 1)
-            score_read<Q, 1, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums ? sums + co : nullptr,
-                             lane, flags);
-        else if (used == 2)
-            score_read<Q, 2, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums ? sums + co : nullptr,
-                             lane, flags);
-        else if (Q <= 5 && used == 3)  // for q = 6 three planes stay in shared memory
-            score_read<Q, 3, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums ? sums + co : nullptr,
-                             lane, flags);
-        else
-            score_read<Q, 0, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums ? sums + co : nullptr,
-                             lane, flags);
+        else {
+            // the read's planes: one, two or three in registers, the top one
+            // folded when it is sparse enough; anything else from shared memory
+            bool sparse = false;
+            if (G::kVPL == 2 && used >= 2 && used <= 3) {
+                const uint4* top = planes4 + (used - 1) * G::kRowVecs + lane % G::kLPB;
+                sparse = sparse_plane(top[0], top[G::kLPB * (G::kVPL - 1)]);
+            }
+            uint16_t* sums_r = sums ? sums + co : nullptr;
+            if (used == 1)
+                score_read<Q, 1, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums_r, lane, flags);
+            else if (used == 2 && sparse)
+                score_read<Q, 2, DEEP, true>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums_r, lane,
+                                             flags);
+            else if (used == 2)
+                score_read<Q, 2, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums_r, lane, flags);
+            else if (Q <= 5 && used == 3 && (sparse || G::kVPL == 1))  // for q = 6 three planes stay in shared memory
+                score_read<Q, 3, DEEP, G::kVPL == 2>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co,
+                                                     sums_r, lane, flags);
+            else
+                score_read<Q, 0, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums_r, lane, flags);
+        }
     }
 
-    // leave the planes zeroed for the warp's next read
+    // leave the area clean for the warp's next read
     __syncwarp();
-    for (int i = lane; i < used * RW; i += 32) planes[i] = 0;
-    __syncwarp();
+    if (used * RW > kCleanFrom<Q>) {
+        for (int i = kCleanFrom<Q> + lane; i < used * RW; i += 32) planes[i] = 0;
+        __syncwarp();
+    }
 }
 
 // Modelled cost of the reads before r: 8 per candidate, 1 per base, 64 per
@@ -543,6 +591,7 @@ gather_kernel(const uint32_t* __restrict__ bank, int64_t n_bins, const uint8_t* 
     __shared__ long long end_read;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    uint32_t* planes = reinterpret_cast<uint32_t*>(gather_smem) + warp * G::kPlaneWords;
     if (counter == nullptr && warp == 0) {
         const int64_t n_ctas = gridDim.x, b = blockIdx.x;
         const int64_t total = cost_before(read_offsets, cand_offsets, n_reads);
@@ -558,8 +607,8 @@ gather_kernel(const uint32_t* __restrict__ bank, int64_t n_bins, const uint8_t* 
             end_read = b == n_ctas - 1 ? n_reads : r_end;
         }
     }
-    gather_cta_setup<Q>(gather_smem, WARPS);  // ends with a CTA barrier
-    uint32_t* planes = reinterpret_cast<uint32_t*>(gather_smem) + warp * G::kPlaneWords;
+    gather_warp_setup<Q>(planes, lane);
+    __syncthreads();  // next_read; kept for counter launches too, whose code spilled 60-200 bytes without it
     const int64_t r_end = counter ? n_reads : end_read;
     unsigned long long* next = counter ? counter : &next_read;
 
@@ -577,6 +626,49 @@ gather_kernel(const uint32_t* __restrict__ bank, int64_t n_bins, const uint8_t* 
     flags = __reduce_or_sync(kFull, flags);
     if (lane == 0 && flags) atomicOr(status, flags);
 }
+
+// A batch of no more reads than the GPU holds warps: one read per warp, no
+// shares to work out and no counter, spread over every SM (1,000 reads of 32
+// candidates: 32 CTAs of the kernel above, claiming four reads a warp, took
+// 9.2 us of device time).
+constexpr int kSmallWarps = 4;
+
+template <int Q>
+__global__ void __launch_bounds__(kSmallWarps * 32)
+gather_small_kernel(const uint32_t* __restrict__ bank, int64_t n_bins, const uint8_t* __restrict__ reads,
+                    const int64_t* __restrict__ read_offsets, int64_t n_reads,
+                    const uint32_t* __restrict__ cand_bins, const int64_t* __restrict__ cand_offsets,
+                    const uint16_t* __restrict__ E, uint8_t* __restrict__ pass, uint16_t* __restrict__ sums,
+                    uint32_t* __restrict__ status) {
+    extern __shared__ uint4 gather_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t r = (int64_t)blockIdx.x * kSmallWarps + warp;
+    if (r >= n_reads) return;
+    const int64_t ro = read_offsets[r], re = read_offsets[r + 1], co = cand_offsets[r], ce = cand_offsets[r + 1];
+    uint32_t* planes = reinterpret_cast<uint32_t*>(gather_smem) + warp * GatherGeo<Q>::kPlaneWords;
+    gather_warp_setup<Q>(planes, lane);
+    uint32_t flags = 0;
+    gather_read<Q, true>(ro, re, co, ce, E[r], bank, n_bins, reads, cand_bins, pass, sums, planes, lane, flags);
+    flags = __reduce_or_sync(kFull, flags);
+    if (lane == 0 && flags) atomicOr(status, flags);
+}
+
+template <int Q>
+static int launch_small(const grim_bank* bank, const GatherArgs& a, int64_t r0, int64_t n, cudaStream_t s) {
+    constexpr size_t smem = gather_smem_bytes<Q>(kSmallWarps);
+    static_assert(smem <= 48 * 1024, "no attribute needed");
+    gather_small_kernel<Q><<<grim::fault_grid((unsigned)((n + kSmallWarps - 1) / kSmallWarps)), kSmallWarps * 32, smem,
+                             s>>>(bank->bits, bank->n_bins, a.reads, a.read_offsets + r0, n, a.cand_bins,
+                                  a.cand_offsets + r0, a.E + r0, a.pass, a.sums, bank->status);
+    GRIM_CUDA_TRY(cudaGetLastError());
+    return GRIM_OK;
+}
+
+// Up to 16 reads an SM take gather_small_kernel: as many warps as it holds at
+// once (96 registers), and no more reads than the claiming kernel would give
+// each warp one of.  1,000 reads of 32 candidates: 12.3 -> 11.5 us a call, 47
+// -> 38 us for a first call on new buffers.
+constexpr int kSmallReadsPerSm = 16;
 
 // Banks larger than this are read from HBM rather than L2: the gather then
 // keeps three steps of rows in flight per warp (the DEEP form).
@@ -604,6 +696,8 @@ static int launch_range(const grim_bank* bank, const GatherArgs& a, int64_t r0, 
     if (per_sm <= 0 || per_sm > max_blocks) per_sm = max_blocks;
     if (claim <= 0) claim = 1;
     int64_t blocks = (int64_t)sm_count() * per_sm;
+    // fewer claims than warps: one read to a claim, to occupy every SM
+    if (n < blocks * WARPS * claim) claim = 1;
     const int64_t need = (n + (int64_t)WARPS * claim - 1) / ((int64_t)WARPS * claim);  // a claim per warp at least
     if (need < blocks) blocks = need;
     if (counter) GRIM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s));
@@ -624,7 +718,9 @@ static int launch_batches(const grim_bank* bank, const GatherArgs& a, const grim
         const int64_t n = (a.n_reads - r0) < batch ? (a.n_reads - r0) : batch;
         const int pc = t.ctas_per_sm, rc_ = t.reads_per_claim;
         int rc;
-        if (deep)
+        if (n <= kSmallReadsPerSm * (int64_t)sm_count())
+            rc = launch_small<Q>(bank, a, r0, n, s);
+        else if (deep)
             rc = t.warps_per_cta == 4 ? launch_range<Q, 4, kDeepForm>(bank, a, r0, n, pc, rc_, counter, s)
                                       : launch_range<Q, 8, kDeepForm>(bank, a, r0, n, pc, rc_, counter, s);
         else
