@@ -166,6 +166,15 @@ int grim_filter_auto(const grim_bank* bank, const uint8_t* reads, const int64_t*
     auto flush = [&](int64_t r_end) -> int {
         if (run0 < 0) return GRIM_OK;
         const int64_t n = r_end - run0;
+        // by bank segment where that is the faster form
+        const int64_t checks = bounds[(size_t)((r_end + batch_reads - 1) / batch_reads)] -
+                               bounds[(size_t)(run0 / batch_reads)];
+        const grim::GatherArgs a{reads, read_offsets + run0, n, cand_bins, cand_offsets + run0, E + run0, pass, nullptr};
+        const int rb = grim::launch_gather_blocked(bank, a, checks, s);
+        if (rb != grim::kBlockedNotBetter && rb != grim::kBlockedNoMemory) {
+            run0 = -1;
+            return rb;
+        }
         t.batch_reads = n;
         const int r = grim_filter_batched(bank, reads, read_offsets + run0, n, cand_bins, cand_offsets + run0,
                                           E + run0, pass, nullptr, &t, stream);

@@ -163,7 +163,7 @@ struct Stream {
 };
 
 __device__ __forceinline__ uint32_t window_id(const uint32_t* __restrict__ cands, int c, int n) {
-    return c < n ? __ldg(cands + c) : 0xFFFFFFFFu;
+    return c < n ? __ldcs(cands + c) : 0xFFFFFFFFu;
 }
 
 // Asks the L2 for the 128-byte lines of a row that will be scored later
@@ -343,7 +343,7 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
             const bool in_range = id < n_bins32;
             if (!in_range) flags |= GRIM_FLAG_BAD_BIN;
             const uint32_t sum = in_range ? red.total : 0u;
-            pass[c] = (in_range && (int)sum >= T) ? 1 : 0;
+            __stcs(pass + c, (uint8_t)((in_range && (int)sum >= T) ? 1 : 0));
             if (sums) sums[c] = (uint16_t)sum;
         }
         st.win_cur = st.win_next;
@@ -423,6 +423,47 @@ __device__ __forceinline__ void gather_warp_setup(uint32_t* planes, int lane) {
     __syncwarp();
 }
 
+// Steps 1-2: the count planes of a read of n_tok token positions; returns how
+// many there are.  Whole warp; bad_base collects codes > 3.
+template <int Q>
+__device__ __forceinline__ int build_planes(const uint8_t* __restrict__ rd, int L, int n_tok,
+                                            uint32_t* __restrict__ planes, int lane, uint32_t& bad_base) {
+    constexpr int RW = GatherGeo<Q>::kRowWords;
+    // byte counters, then the planes from them (q <= 5); for q = 6 the 4096
+    // counters cost more to cut into planes than the carries they save
+    if (Q <= 5 && n_tok <= 255) {
+        for_each_token5<Q>(rd, L, lane, bad_base,
+                           [&](uint32_t tok) { atomicAdd(&planes[counter_word<Q>(tok)], 1u << (tok & 0x18u)); });
+        __syncwarp();
+        return planes_from_counters<Q>(planes, lane);
+    }
+    // q = 6 and longer reads: a carry chain of atomicXor per token
+    for (int i = lane; i < kCleanFrom<Q>; i += 32) planes[i] = 0;
+    __syncwarp();
+    int top = -1;  // highest plane this lane set
+    for_each_token5<Q>(rd, L, lane, bad_base, [&](uint32_t tok) {
+        const uint32_t w = tok >> 5, m = 1u << (tok & 31);
+        int p = 0;
+        while (p < kPlanes) {
+            const uint32_t old = atomicXor(&planes[p * RW + w], m);
+            if (!(old & m)) break;
+            ++p;
+        }
+        top = p > top ? p : top;
+    });
+    return (int)__reduce_max_sync(kFull, (unsigned)(top + 1));
+}
+
+// The plane area clean again after a read of `used` planes.
+template <int Q>
+__device__ __forceinline__ void clean_planes(uint32_t* __restrict__ planes, int used, int lane) {
+    __syncwarp();
+    if (used * GatherGeo<Q>::kRowWords > kCleanFrom<Q>) {
+        for (int i = kCleanFrom<Q> + lane; i < used * GatherGeo<Q>::kRowWords; i += 32) planes[i] = 0;
+        __syncwarp();
+    }
+}
+
 // The whole filter for read r, by one warp (steps 0-5 above).  The warp's
 // plane area is zero from kCleanFrom on at entry, and left so.
 // ro, re: the read's bases; co, ce: its candidates; e: its edit budget.
@@ -434,7 +475,6 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
                                             uint16_t* __restrict__ sums, uint32_t* __restrict__ planes, int lane,
                                             uint32_t& flags) {
     using G = GatherGeo<Q>;
-    constexpr int RW = G::kRowWords;
     const uint4* planes4 = reinterpret_cast<const uint4*>(planes);
     if (ce < co) {  // nothing sensible to write for this read
         flags |= GRIM_FLAG_BAD_OFFSETS;
@@ -462,31 +502,8 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
 
     // 1-2. tokens into bit-sliced count planes
     uint32_t bad_base = 0;
-    int used;
     const int n_tok = L - Q + 1 > 0 ? L - Q + 1 : 0;
-    // byte counters, then the planes from them (q <= 5); for q = 6 the 4096
-    // counters cost more to cut into planes than the carries they save
-    if (Q <= 5 && n_tok <= 255) {
-        for_each_token5<Q>(rd, L, lane, bad_base,
-                           [&](uint32_t tok) { atomicAdd(&planes[counter_word<Q>(tok)], 1u << (tok & 0x18u)); });
-        __syncwarp();
-        used = planes_from_counters<Q>(planes, lane);
-    } else {  // q = 6 and longer reads: a carry chain of atomicXor per token
-        for (int i = lane; i < kCleanFrom<Q>; i += 32) planes[i] = 0;
-        __syncwarp();
-        int top = -1;  // highest plane this lane set
-        for_each_token5<Q>(rd, L, lane, bad_base, [&](uint32_t tok) {
-            const uint32_t w = tok >> 5, m = 1u << (tok & 31);
-            int p = 0;
-            while (p < kPlanes) {
-                const uint32_t old = atomicXor(&planes[p * RW + w], m);
-                if (!(old & m)) break;
-                ++p;
-            }
-            top = p > top ? p : top;
-        });
-        used = (int)__reduce_max_sync(kFull, (unsigned)(top + 1));
-    }
+    const int used = build_planes<Q>(rd, L, n_tok, planes, lane, bad_base);
     if (__any_sync(kFull, bad_base)) {
         flags |= GRIM_FLAG_BAD_BASE;
         bad_read = true;
@@ -522,12 +539,7 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
         }
     }
 
-    // leave the area clean for the warp's next read
-    __syncwarp();
-    if (used * RW > kCleanFrom<Q>) {
-        for (int i = kCleanFrom<Q> + lane; i < used * RW; i += 32) planes[i] = 0;
-        __syncwarp();
-    }
+    clean_planes<Q>(planes, used, lane);  // for the warp's next read
 }
 
 // Modelled cost of the reads before r: 8 per candidate, 1 per base, 64 per
@@ -706,6 +718,307 @@ static int launch_range(const grim_bank* bank, const GatherArgs& a, int64_t r0, 
         a.pass, a.sums, bank->status, claim, counter);
     GRIM_CUDA_TRY(cudaGetLastError());
     return GRIM_OK;
+}
+
+// ------------------------------------------------------------ by bank segment
+
+// A bank beyond the L2 whose rows are scored many times over (3.1 Gbp, 1M
+// reads of ~1,700 candidates: 138 checks a row) is read from HBM once per
+// check by the kernels above.  Here the checks go segment by segment of the
+// bank (64 MB, about half the L2), all reads' candidates in one segment before
+// the next, so that a segment comes from HBM once and its rows from the L2:
+//   1. blocked_prep_kernel (warp per read): the read's count planes and
+//      threshold to memory, and where each segment's candidates start in its
+//      list.  Lists ascend as seed tables give them; one that does not is cut
+//      at other places and only loses the order (every candidate is scored by
+//      its own id whatever segment it was counted to).  A read that is
+//      invalid or has no or more than two planes is listed for step 3;
+//   2. blocked_kernel: warps claim (segment, 32 reads) in segment order; the
+//      next read's planes (cp.async) and candidate ids come in while one is
+//      scored;
+//   3. blocked_direct_kernel: the listed reads as in gather_kernel.
+// 3.1 Gbp, 1M reads, 1.67e9 checks: 38.2 -> 25.3 ms, of which the ordering
+// (step 1) is 1.25.  Bound: rows from the L2 (8.8 TB/s of the 14 a sequential
+// read of it reaches).  Segments of 32 MB 29.9 (half as many candidates per
+// read and segment), of 128 MB 27.9; 3 CTAs of 8 warps 26.4; two row buffers
+// and 4 CTAs 27.3.
+constexpr size_t kSegmentBytes = size_t(64) << 20;
+// Where the line lies (q = 5, reads of 100 bases unless said; by segment
+// against the claiming kernel, ms): rows of 8 GB read in all - 3.1 Gbp 30,000
+// reads (6.4 GB) 1.18 / 1.18, 60,000 1.95 / 2.23, 120,000 3.28 / 4.35, 1M 25.3
+// / 37.9; 1 Gbp 60,000 (4 GB) 0.71 / 0.69, 200,000 1.77 / 2.14; 600 Mbp 400,000
+// 2.13 / 2.42.  Banks of 200 MB are half in the L2 already: 0.50 / 0.42.  At
+// least 20 candidates of a read in a segment, or the switches between reads
+// cost more: 24 (reads of 36 bases) 3.84 / 4.20, 16 (24 bases) 4.27 / 3.78.
+// q = 6 rows are slower this way (100 Mbp: 11.4 / 9.7) and are left as above.
+constexpr double kBlockedBankBytes = 256e6;
+constexpr double kBlockedRowBytes = 8e9;
+constexpr int64_t kBlockedChecksPerItem = 20;
+constexpr int kMaxSegments = 256;
+constexpr int64_t kBlockedReads = int64_t(1) << 20;  // reads per round over the bank
+
+struct BlockedRead {
+    int T;
+    int mode;  // 0: two planes, the upper one folded (row_sum8); 1: two planes
+};
+
+template <int Q>
+__global__ void __launch_bounds__(kSmallWarps * 32)
+blocked_prep_kernel(const uint8_t* __restrict__ reads, const int64_t* __restrict__ read_offsets, int64_t n_reads,
+                    const uint32_t* __restrict__ cand_bins, const int64_t* __restrict__ cand_offsets,
+                    const uint16_t* __restrict__ E, int seg_shift, int n_seg,
+                    uint4* __restrict__ planes_out, BlockedRead* __restrict__ info, uint32_t* __restrict__ starts,
+                    uint32_t* __restrict__ list, uint32_t* __restrict__ n_list) {
+    using G = GatherGeo<Q>;
+    extern __shared__ uint4 gather_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t* planes = reinterpret_cast<uint32_t*>(gather_smem) + warp * G::kPlaneWords;
+    const uint4* planes4 = reinterpret_cast<const uint4*>(planes);
+    gather_warp_setup<Q>(planes, lane);
+    for (int64_t r = (int64_t)blockIdx.x * kSmallWarps + warp; r < n_reads; r += (int64_t)gridDim.x * kSmallWarps) {
+        const int64_t ro = read_offsets[r], re = read_offsets[r + 1], co = cand_offsets[r], ce = cand_offsets[r + 1];
+        bool direct = ce < co || ce - co > 0x7fffffff || re < ro || re - ro > GRIM_MAX_READ_LEN;
+        const int n_c = direct ? 0 : (int)(ce - co);
+        if (!direct) {
+            const int L = (int)(re - ro), n_tok = L - Q + 1 > 0 ? L - Q + 1 : 0;
+            uint32_t bad_base = 0;
+            const int used = build_planes<Q>(reads + ro, L, n_tok, planes, lane, bad_base);
+            direct = __any_sync(kFull, bad_base) || (n_c > 0 && (used < 1 || used > 2));
+            __syncwarp();
+            if (!direct && n_c > 0) {
+                const uint4 zero = make_uint4(0, 0, 0, 0);
+                uint4 top[G::kVPL];
+#pragma unroll
+                for (int u = 0; u < G::kVPL; u++)
+                    top[u] = used == 2 ? planes4[G::kRowVecs + lane % G::kLPB + u * G::kLPB] : zero;
+                const bool sparse = sparse_plane(top[0], top[G::kVPL - 1]);
+                for (int v = lane; v < 2 * G::kRowVecs; v += 32)
+                    planes_out[r * 2 * G::kRowVecs + v] = v < G::kRowVecs || used == 2 ? planes4[v] : zero;
+                if (lane == 0) info[r] = BlockedRead{n_tok - Q * (int)E[r], sparse ? 0 : 1};
+            }
+            clean_planes<Q>(planes, used, lane);
+        }
+        // where each segment's candidates start: a search among 32 samples of
+        // the list, then in the stretch between two of them
+        const uint32_t* cands = cand_bins + co;
+        const uint32_t sample = n_c > 0 ? __ldg(cands + (int)((int64_t)lane * n_c >> 5)) : 0u;
+        uint32_t before = 0;
+        for (int s0 = 0; s0 <= n_seg; s0 += 32) {
+            const int sg = s0 + lane;
+            const uint32_t key = (uint32_t)sg << seg_shift;  // sg < n_seg: below n_bins
+            int lo = 0, hi = 32;  // samples below key: a prefix of an ascending list
+#pragma unroll
+            for (int step = 0; step < 5; step++) {
+                const int mid = (lo + hi) >> 1;
+                if (__shfl_sync(kFull, sample, mid) < key) lo = mid;
+                else hi = mid;
+            }
+            uint32_t at = 0;
+            if (sg >= n_seg) {
+                at = (uint32_t)n_c;
+            } else if (sg > 0 && n_c > 0) {
+                int a = (int)((int64_t)lo * n_c >> 5), z = hi < 32 ? (int)((int64_t)hi * n_c >> 5) : n_c;
+                while (a < z) {
+                    const int mid = (a + z) >> 1;
+                    if (__ldg(cands + mid) < key) a = mid + 1;
+                    else z = mid;
+                }
+                at = (uint32_t)a;
+            }
+            // in an unordered list the places found need not ascend
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, at, o);
+                if (lane >= o) at = y > at ? y : at;
+            }
+            at = before > at ? before : at;
+            before = __shfl_sync(kFull, at, 31);
+            if (sg <= n_seg) starts[(int64_t)sg * n_reads + r] = direct ? 0u : at;
+        }
+        if (direct && lane == 0) list[atomicAdd(n_list, 1u)] = (uint32_t)r;
+        __syncwarp();
+    }
+}
+
+constexpr int kBlockedWarps = 4;
+constexpr int kBlockedCtas = 7;  // per SM (72 registers)
+
+template <int Q>
+__global__ void __launch_bounds__(kBlockedWarps * 32, kBlockedCtas)
+blocked_kernel(const uint32_t* __restrict__ bank, uint32_t n_bins32, const uint32_t* __restrict__ cand_bins,
+               const int64_t* __restrict__ cand_offsets, int64_t n_reads, int n_seg,
+               const uint4* __restrict__ planes_in, const BlockedRead* __restrict__ info,
+               const uint32_t* __restrict__ starts, uint8_t* __restrict__ pass, uint32_t* __restrict__ status,
+               unsigned long long* __restrict__ counter) {
+    using G = GatherGeo<Q>;
+    using S = Stream<Q, true>;
+    constexpr int kVecs = 2 * G::kRowVecs;  // two planes
+    __shared__ uint4 planes_s[kBlockedWarps][2][kVecs];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s = lane % G::kLPB, g = lane / G::kLPB;
+    const int64_t groups = (n_reads + 31) >> 5, total = groups * n_seg;
+    uint32_t flags = 0;
+    while (true) {
+        unsigned long long item = 0;
+        if (lane == 0) item = atomicAdd(counter, 1ull);
+        item = __shfl_sync(kFull, item, 0);
+        if ((int64_t)item >= total) break;
+        const int64_t sg = (int64_t)item / groups, r0 = ((int64_t)item - sg * groups) << 5;
+        // lane i: read r0 + i's candidates in this segment
+        int64_t first = 0;
+        int n_l = 0;
+        BlockedRead rd{0, 0};
+        if (r0 + lane < n_reads) {
+            const uint32_t lo = __ldg(starts + sg * n_reads + r0 + lane);
+            n_l = (int)(__ldg(starts + (sg + 1) * n_reads + r0 + lane) - lo);
+            if (n_l > 0) {
+                first = __ldg(cand_offsets + r0 + lane) + lo;
+                rd = info[r0 + lane];
+            }
+        }
+        uint32_t todo = __ballot_sync(kFull, n_l > 0);
+        if (todo == 0) continue;
+        int i = __ffs(todo) - 1, buf = 0;
+        auto ask_planes = [&](int which, int b) {
+            const uint4* src = planes_in + (r0 + which) * kVecs;
+#pragma unroll
+            for (int v = lane; v < kVecs; v += 32)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
+                                 (uint32_t)__cvta_generic_to_shared(&planes_s[warp][b][v])),
+                             "l"(src + v)
+                             : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        ask_planes(i, 0);
+        int64_t at = __shfl_sync(kFull, first, i);
+        int n = __shfl_sync(kFull, n_l, i);
+        uint32_t id0 = window_id(cand_bins + at, lane, n), id1 = window_id(cand_bins + at, 32 + lane, n);
+        while (true) {
+            const int64_t at_now = at;
+            const int n_now = n, i_now = i;
+            S st;
+            st.win_cur = id0;
+            st.win_next = id1;
+#pragma unroll
+            for (int k = 0; k < S::kAhead; k++) {
+                const int idx = k * G::kBPS + g;
+                const uint32_t id = __shfl_sync(kFull, idx < 32 ? st.win_cur : st.win_next, idx & 31);
+                fetch_row<Q>(st.r[k], id, bank, n_bins32, s);
+            }
+            todo &= todo - 1;
+            if (todo) {  // the next read's planes and ids
+                i = __ffs(todo) - 1;
+                ask_planes(i, buf ^ 1);
+                at = __shfl_sync(kFull, first, i);
+                n = __shfl_sync(kFull, n_l, i);
+                id0 = window_id(cand_bins + at, lane, n);
+                id1 = window_id(cand_bins + at, 32 + lane, n);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncwarp();
+            const int T = __shfl_sync(kFull, rd.T, i_now);
+            if (__shfl_sync(kFull, rd.mode, i_now) == 0)
+                score_read<Q, 2, true, true>(st, planes_s[warp][buf], 2, T, n_now, cand_bins + at_now, bank, n_bins32,
+                                             pass + at_now, nullptr, lane, flags);
+            else
+                score_read<Q, 2, true>(st, planes_s[warp][buf], 2, T, n_now, cand_bins + at_now, bank, n_bins32,
+                                       pass + at_now, nullptr, lane, flags);
+            __syncwarp();
+            if (!todo) break;
+            buf ^= 1;
+        }
+    }
+    flags = __reduce_or_sync(kFull, flags);
+    if (lane == 0 && flags) atomicOr(status, flags);
+}
+
+template <int Q>
+__global__ void __launch_bounds__(kSmallWarps * 32, 5)
+blocked_direct_kernel(const uint32_t* __restrict__ bank, int64_t n_bins, const uint8_t* __restrict__ reads,
+                      const int64_t* __restrict__ read_offsets, const uint32_t* __restrict__ cand_bins,
+                      const int64_t* __restrict__ cand_offsets, const uint16_t* __restrict__ E,
+                      uint8_t* __restrict__ pass, uint32_t* __restrict__ status, const uint32_t* __restrict__ list,
+                      const uint32_t* __restrict__ n_list, uint32_t* __restrict__ next) {
+    extern __shared__ uint4 gather_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t* planes = reinterpret_cast<uint32_t*>(gather_smem) + warp * GatherGeo<Q>::kPlaneWords;
+    gather_warp_setup<Q>(planes, lane);
+    const uint32_t n = *n_list;
+    uint32_t flags = 0;
+    while (true) {
+        uint32_t i = 0;
+        if (lane == 0) i = atomicAdd(next, 1u);
+        i = __shfl_sync(kFull, i, 0);
+        if (i >= n) break;
+        const uint32_t r = list[i];
+        gather_read<Q, true>(read_offsets[r], read_offsets[r + 1], cand_offsets[r], cand_offsets[r + 1], E[r], bank,
+                             n_bins, reads, cand_bins, pass, nullptr, planes, lane, flags);
+    }
+    flags = __reduce_or_sync(kFull, flags);
+    if (lane == 0 && flags) atomicOr(status, flags);
+}
+
+template <int Q>
+static int launch_blocked(const grim_bank* bank, const GatherArgs& a, int seg_shift, int n_seg, cudaStream_t s) {
+    using G = GatherGeo<Q>;
+    const int64_t most = a.n_reads < kBlockedReads ? a.n_reads : kBlockedReads;
+    const size_t planes_bytes = (size_t)most * 2 * G::kRowVecs * 16, info_bytes = (size_t)most * sizeof(BlockedRead);
+    const size_t starts_bytes = ((size_t)(n_seg + 1) * most * 4 + 15) & ~(size_t)15;
+    uint8_t* mem = nullptr;
+    const cudaError_t ea = scratch_alloc((void**)&mem, 64 + planes_bytes + info_bytes + starts_bytes + most * 4, s);
+    if (ea != cudaSuccess) {
+        cudaGetLastError();
+        return kBlockedNoMemory;
+    }
+    unsigned long long* counter = reinterpret_cast<unsigned long long*>(mem);
+    uint32_t *n_list = reinterpret_cast<uint32_t*>(mem + 8), *next = n_list + 1;
+    uint4* planes = reinterpret_cast<uint4*>(mem + 64);
+    BlockedRead* info = reinterpret_cast<BlockedRead*>(mem + 64 + planes_bytes);
+    uint32_t* starts = reinterpret_cast<uint32_t*>(mem + 64 + planes_bytes + info_bytes);
+    uint32_t* list = reinterpret_cast<uint32_t*>(mem + 64 + planes_bytes + info_bytes + starts_bytes);
+    constexpr size_t smem = gather_smem_bytes<Q>(kSmallWarps);
+    cudaError_t e = cudaSuccess;
+    for (int64_t r0 = 0; r0 < a.n_reads && e == cudaSuccess; r0 += most) {
+        const int64_t n = a.n_reads - r0 < most ? a.n_reads - r0 : most;
+        e = cudaMemsetAsync(mem, 0, 64, s);
+        if (e != cudaSuccess) break;
+        const int64_t need = (n + kSmallWarps - 1) / kSmallWarps, wave = (int64_t)sm_count() * 12;
+        blocked_prep_kernel<Q><<<fault_grid((unsigned)(need < wave ? need : wave)), kSmallWarps * 32, smem, s>>>(
+            a.reads, a.read_offsets + r0, n, a.cand_bins, a.cand_offsets + r0, a.E + r0,
+            seg_shift, n_seg, planes, info, starts, list, n_list);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) break;
+        blocked_kernel<Q><<<fault_grid((unsigned)(sm_count() * kBlockedCtas)), kBlockedWarps * 32, 0, s>>>(
+            bank->bits, (uint32_t)bank->n_bins, a.cand_bins, a.cand_offsets + r0, n, n_seg, planes, info, starts,
+            a.pass, bank->status, counter);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) break;
+        blocked_direct_kernel<Q><<<fault_grid((unsigned)(sm_count() * 4)), kSmallWarps * 32, smem, s>>>(
+            bank->bits, bank->n_bins, a.reads, a.read_offsets + r0, a.cand_bins, a.cand_offsets + r0, a.E + r0, a.pass,
+            bank->status, list, n_list, next);
+        e = cudaGetLastError();
+    }
+    cudaFreeAsync(mem, s);
+    if (e != cudaSuccess) {
+        set_last_cuda_error(e);
+        return GRIM_ECUDA;
+    }
+    return GRIM_OK;
+}
+
+int launch_gather_blocked(const grim_bank* bank, const GatherArgs& a, int64_t n_checks, cudaStream_t s) {
+    const int64_t row_bytes = bank->row_words * 4;
+    if (bank->q != 5 || a.sums || (double)bank->n_bins * (double)row_bytes < kBlockedBankBytes)
+        return kBlockedNotBetter;
+    int seg_shift = 0;
+    while ((row_bytes << (seg_shift + 1)) <= (int64_t)kSegmentBytes) seg_shift++;
+    const int64_t n_seg = (bank->n_bins + (int64_t(1) << seg_shift) - 1) >> seg_shift;
+    if (n_seg > kMaxSegments || (double)n_checks * (double)row_bytes < kBlockedRowBytes ||
+        n_checks < kBlockedChecksPerItem * n_seg * a.n_reads)
+        return kBlockedNotBetter;
+    return launch_blocked<5>(bank, a, seg_shift, (int)n_seg, s);
 }
 
 template <int Q>

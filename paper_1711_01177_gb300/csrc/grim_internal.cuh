@@ -112,6 +112,12 @@ struct GatherArgs {
 int launch_gather_batches(const grim_bank* bank, const GatherArgs& a, const grim_tune& t,
                           unsigned long long* counter, cudaStream_t stream);
 
+// The same pass bytes (a.sums null) with the checks ordered by bank segment:
+// for banks beyond the L2 whose rows are scored many times (n_checks in all).
+// Besides status codes: kBlockedNotBetter / kBlockedNoMemory, nothing done.
+constexpr int kBlockedNotBetter = -1, kBlockedNoMemory = -2;
+int launch_gather_blocked(const grim_bank* bank, const GatherArgs& a, int64_t n_checks, cudaStream_t stream);
+
 size_t scan_scratch_bytes(int q, int64_t n_reads);
 // Whether grim_scan_noalloc takes that many reads (the header's formula).
 bool scan_noalloc_admits(int q, int64_t n_reads);
