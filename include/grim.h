@@ -329,7 +329,7 @@ int grim_choose_form(const grim_bank* bank, int64_t n_reads, int64_t n_checks, i
  * consecutive gathered batches is one launch, or, with q = 5, a bank beyond
  * the L2 and rows scored many times over, three launches per 2^20 reads that
  * take the candidates segment by segment of the bank (faster for ascending
- * lists; about 270 bytes and 4 per 64 MB of bank of the library's pool for
+ * lists; about 300 bytes and 4 per 72 MB of bank of the library's pool for
  * each of those reads, and the one launch where it has none).  Reads every
  * batch's
  * candidate count from the device up front (synchronising `stream` once,

@@ -725,14 +725,15 @@ static int launch_range(const grim_bank* bank, const GatherArgs& a, int64_t r0, 
 // A bank beyond the L2 whose rows are scored many times over (3.1 Gbp, 1M
 // reads of ~1,700 candidates: 138 checks a row) is read from HBM once per
 // check by the kernels above.  Here the checks go segment by segment of the
-// bank (64 MB, about half the L2), all reads' candidates in one segment before
+// bank (72 MB, about half the L2), all reads' candidates in one segment before
 // the next, so that a segment comes from HBM once and its rows from the L2:
 //   1. blocked_prep_kernel (warp per read): the read's count planes and
 //      threshold to memory, and where each segment's candidates start in its
 //      list.  Lists ascend as seed tables give them; one that does not is cut
 //      at other places and only loses the order (every candidate is scored by
 //      its own id whatever segment it was counted to).  A read that is
-//      invalid or has no or more than two planes is listed for step 3;
+//      invalid or has no or more than four planes is listed for step 3 (one
+//      such read is a serial tail of 0.2 ms: its rows come from HBM);
 //   2. blocked_kernel: warps claim (segment, 32 reads) in segment order; the
 //      next read's planes (cp.async) and candidate ids come in while one is
 //      scored;
@@ -742,7 +743,7 @@ static int launch_range(const grim_bank* bank, const GatherArgs& a, int64_t r0, 
 // read of it reaches).  Segments of 32 MB 29.9 (half as many candidates per
 // read and segment), of 128 MB 27.9; 3 CTAs of 8 warps 26.4; two row buffers
 // and 4 CTAs 27.3.
-constexpr size_t kSegmentBytes = size_t(64) << 20;
+constexpr size_t kSegmentBytes = size_t(72) << 20;
 // Where the line lies (q = 5, reads of 100 bases unless said; by segment
 // against the claiming kernel, ms): rows of 8 GB read in all - 3.1 Gbp 30,000
 // reads (6.4 GB) 1.18 / 1.18, 60,000 1.95 / 2.23, 120,000 3.28 / 4.35, 1M 25.3
@@ -759,16 +760,18 @@ constexpr int64_t kBlockedReads = int64_t(1) << 20;  // reads per round over the
 
 struct BlockedRead {
     int T;
-    int mode;  // 0: two planes, the upper one folded (row_sum8); 1: two planes
+    int mode;  // 0: two planes, the upper one folded (row_sum8); 1: two planes; 2 + i: four, two of them in extra[i]
 };
+constexpr int kExtraShare = 16;  // one read in so many may have three or four planes
 
 template <int Q>
 __global__ void __launch_bounds__(kSmallWarps * 32)
 blocked_prep_kernel(const uint8_t* __restrict__ reads, const int64_t* __restrict__ read_offsets, int64_t n_reads,
                     const uint32_t* __restrict__ cand_bins, const int64_t* __restrict__ cand_offsets,
-                    const uint16_t* __restrict__ E, int seg_shift, int n_seg,
-                    uint4* __restrict__ planes_out, BlockedRead* __restrict__ info, uint32_t* __restrict__ starts,
-                    uint32_t* __restrict__ list, uint32_t* __restrict__ n_list) {
+                    const uint16_t* __restrict__ E, uint32_t seg_bins, int n_seg,
+                    uint4* __restrict__ planes_out, uint4* __restrict__ extra, uint32_t n_extra,
+                    BlockedRead* __restrict__ info, uint32_t* __restrict__ starts, uint32_t* __restrict__ list,
+                    uint32_t* __restrict__ counts) {  // counts[0]: list's length, counts[2]: extra's
     using G = GatherGeo<Q>;
     extern __shared__ uint4 gather_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -783,18 +786,28 @@ blocked_prep_kernel(const uint8_t* __restrict__ reads, const int64_t* __restrict
             const int L = (int)(re - ro), n_tok = L - Q + 1 > 0 ? L - Q + 1 : 0;
             uint32_t bad_base = 0;
             const int used = build_planes<Q>(reads + ro, L, n_tok, planes, lane, bad_base);
-            direct = __any_sync(kFull, bad_base) || (n_c > 0 && (used < 1 || used > 2));
+            direct = __any_sync(kFull, bad_base) || (n_c > 0 && (used < 1 || used > 4));
             __syncwarp();
             if (!direct && n_c > 0) {
-                const uint4 zero = make_uint4(0, 0, 0, 0);
-                uint4 top[G::kVPL];
-#pragma unroll
-                for (int u = 0; u < G::kVPL; u++)
-                    top[u] = used == 2 ? planes4[G::kRowVecs + lane % G::kLPB + u * G::kLPB] : zero;
-                const bool sparse = sparse_plane(top[0], top[G::kVPL - 1]);
+                int mode = 0;
+                if (used > 2) {
+                    uint32_t x = 0;
+                    if (lane == 0) x = atomicAdd(counts + 2, 1u);
+                    x = __shfl_sync(kFull, x, 0);
+                    direct = x >= n_extra;
+                    mode = 2 + (int)x;
+                    if (!direct)
+                        for (int v = lane; v < 2 * G::kRowVecs; v += 32)  // planes 2 and 3
+                            extra[(size_t)x * 2 * G::kRowVecs + v] =
+                                v < G::kRowVecs || used == 4 ? planes4[2 * G::kRowVecs + v] : make_uint4(0, 0, 0, 0);
+                } else {
+                    const uint4* top = planes4 + G::kRowVecs + lane % G::kLPB;
+                    mode = used == 1 || sparse_plane(top[0], top[G::kLPB * (G::kVPL - 1)]) ? 0 : 1;
+                }
                 for (int v = lane; v < 2 * G::kRowVecs; v += 32)
-                    planes_out[r * 2 * G::kRowVecs + v] = v < G::kRowVecs || used == 2 ? planes4[v] : zero;
-                if (lane == 0) info[r] = BlockedRead{n_tok - Q * (int)E[r], sparse ? 0 : 1};
+                    planes_out[r * 2 * G::kRowVecs + v] =
+                        v < G::kRowVecs || used >= 2 ? planes4[v] : make_uint4(0, 0, 0, 0);
+                if (lane == 0) info[r] = BlockedRead{n_tok - Q * (int)E[r], mode};
             }
             clean_planes<Q>(planes, used, lane);
         }
@@ -805,7 +818,7 @@ blocked_prep_kernel(const uint8_t* __restrict__ reads, const int64_t* __restrict
         uint32_t before = 0;
         for (int s0 = 0; s0 <= n_seg; s0 += 32) {
             const int sg = s0 + lane;
-            const uint32_t key = (uint32_t)sg << seg_shift;  // sg < n_seg: below n_bins
+            const uint32_t key = (uint32_t)sg * seg_bins;  // sg < n_seg: below n_bins
             int lo = 0, hi = 32;  // samples below key: a prefix of an ascending list
 #pragma unroll
             for (int step = 0; step < 5; step++) {
@@ -835,7 +848,7 @@ blocked_prep_kernel(const uint8_t* __restrict__ reads, const int64_t* __restrict
             before = __shfl_sync(kFull, at, 31);
             if (sg <= n_seg) starts[(int64_t)sg * n_reads + r] = direct ? 0u : at;
         }
-        if (direct && lane == 0) list[atomicAdd(n_list, 1u)] = (uint32_t)r;
+        if (direct && lane == 0) list[atomicAdd(counts, 1u)] = (uint32_t)r;
         __syncwarp();
     }
 }
@@ -847,13 +860,13 @@ template <int Q>
 __global__ void __launch_bounds__(kBlockedWarps * 32, kBlockedCtas)
 blocked_kernel(const uint32_t* __restrict__ bank, uint32_t n_bins32, const uint32_t* __restrict__ cand_bins,
                const int64_t* __restrict__ cand_offsets, int64_t n_reads, int n_seg,
-               const uint4* __restrict__ planes_in, const BlockedRead* __restrict__ info,
+               const uint4* __restrict__ planes_in, const uint4* __restrict__ extra, const BlockedRead* __restrict__ info,
                const uint32_t* __restrict__ starts, uint8_t* __restrict__ pass, uint32_t* __restrict__ status,
                unsigned long long* __restrict__ counter) {
     using G = GatherGeo<Q>;
     using S = Stream<Q, true>;
     constexpr int kVecs = 2 * G::kRowVecs;  // two planes
-    __shared__ uint4 planes_s[kBlockedWarps][2][kVecs];
+    __shared__ uint4 planes_s[kBlockedWarps][2][2 * kVecs];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int s = lane % G::kLPB, g = lane / G::kLPB;
     const int64_t groups = (n_reads + 31) >> 5, total = groups * n_seg;
@@ -879,14 +892,18 @@ blocked_kernel(const uint32_t* __restrict__ bank, uint32_t n_bins32, const uint3
         uint32_t todo = __ballot_sync(kFull, n_l > 0);
         if (todo == 0) continue;
         int i = __ffs(todo) - 1, buf = 0;
-        auto ask_planes = [&](int which, int b) {
-            const uint4* src = planes_in + (r0 + which) * kVecs;
+        auto ask = [&](uint4* dst, const uint4* src) {
 #pragma unroll
             for (int v = lane; v < kVecs; v += 32)
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
-                                 (uint32_t)__cvta_generic_to_shared(&planes_s[warp][b][v])),
+                                 (uint32_t)__cvta_generic_to_shared(dst + v)),
                              "l"(src + v)
                              : "memory");
+        };
+        auto ask_planes = [&](int which, int b) {
+            ask(planes_s[warp][b], planes_in + (r0 + which) * kVecs);
+            const int mode = __shfl_sync(kFull, rd.mode, which);
+            if (mode >= 2) ask(planes_s[warp][b] + kVecs, extra + (size_t)(mode - 2) * kVecs);
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         ask_planes(i, 0);
@@ -919,11 +936,15 @@ blocked_kernel(const uint32_t* __restrict__ bank, uint32_t n_bins32, const uint3
             }
             __syncwarp();
             const int T = __shfl_sync(kFull, rd.T, i_now);
-            if (__shfl_sync(kFull, rd.mode, i_now) == 0)
+            const int mode = __shfl_sync(kFull, rd.mode, i_now);
+            if (mode == 0)
                 score_read<Q, 2, true, true>(st, planes_s[warp][buf], 2, T, n_now, cand_bins + at_now, bank, n_bins32,
                                              pass + at_now, nullptr, lane, flags);
-            else
+            else if (mode == 1)
                 score_read<Q, 2, true>(st, planes_s[warp][buf], 2, T, n_now, cand_bins + at_now, bank, n_bins32,
+                                       pass + at_now, nullptr, lane, flags);
+            else
+                score_read<Q, 0, true>(st, planes_s[warp][buf], 4, T, n_now, cand_bins + at_now, bank, n_bins32,
                                        pass + at_now, nullptr, lane, flags);
             __syncwarp();
             if (!todo) break;
@@ -961,23 +982,27 @@ blocked_direct_kernel(const uint32_t* __restrict__ bank, int64_t n_bins, const u
 }
 
 template <int Q>
-static int launch_blocked(const grim_bank* bank, const GatherArgs& a, int seg_shift, int n_seg, cudaStream_t s) {
+static int launch_blocked(const grim_bank* bank, const GatherArgs& a, uint32_t seg_bins, int n_seg, cudaStream_t s) {
     using G = GatherGeo<Q>;
     const int64_t most = a.n_reads < kBlockedReads ? a.n_reads : kBlockedReads;
     const size_t planes_bytes = (size_t)most * 2 * G::kRowVecs * 16, info_bytes = (size_t)most * sizeof(BlockedRead);
+    const uint32_t n_extra = (uint32_t)(most / kExtraShare + 32);
+    const size_t extra_bytes = (size_t)n_extra * 2 * G::kRowVecs * 16;
     const size_t starts_bytes = ((size_t)(n_seg + 1) * most * 4 + 15) & ~(size_t)15;
     uint8_t* mem = nullptr;
-    const cudaError_t ea = scratch_alloc((void**)&mem, 64 + planes_bytes + info_bytes + starts_bytes + most * 4, s);
+    const cudaError_t ea = scratch_alloc((void**)&mem, 64 + planes_bytes + extra_bytes + info_bytes + starts_bytes + most * 4, s);
     if (ea != cudaSuccess) {
         cudaGetLastError();
         return kBlockedNoMemory;
     }
     unsigned long long* counter = reinterpret_cast<unsigned long long*>(mem);
-    uint32_t *n_list = reinterpret_cast<uint32_t*>(mem + 8), *next = n_list + 1;
-    uint4* planes = reinterpret_cast<uint4*>(mem + 64);
-    BlockedRead* info = reinterpret_cast<BlockedRead*>(mem + 64 + planes_bytes);
-    uint32_t* starts = reinterpret_cast<uint32_t*>(mem + 64 + planes_bytes + info_bytes);
-    uint32_t* list = reinterpret_cast<uint32_t*>(mem + 64 + planes_bytes + info_bytes + starts_bytes);
+    uint32_t *counts = reinterpret_cast<uint32_t*>(mem + 8), *next = counts + 1;  // counts[0], next, counts[2]
+    uint8_t* p = mem + 64;
+    uint4* planes = reinterpret_cast<uint4*>(p);
+    uint4* extra = reinterpret_cast<uint4*>(p += planes_bytes);
+    BlockedRead* info = reinterpret_cast<BlockedRead*>(p += extra_bytes);
+    uint32_t* starts = reinterpret_cast<uint32_t*>(p += info_bytes);
+    uint32_t* list = reinterpret_cast<uint32_t*>(p += starts_bytes);
     constexpr size_t smem = gather_smem_bytes<Q>(kSmallWarps);
     cudaError_t e = cudaSuccess;
     for (int64_t r0 = 0; r0 < a.n_reads && e == cudaSuccess; r0 += most) {
@@ -987,17 +1012,17 @@ static int launch_blocked(const grim_bank* bank, const GatherArgs& a, int seg_sh
         const int64_t need = (n + kSmallWarps - 1) / kSmallWarps, wave = (int64_t)sm_count() * 12;
         blocked_prep_kernel<Q><<<fault_grid((unsigned)(need < wave ? need : wave)), kSmallWarps * 32, smem, s>>>(
             a.reads, a.read_offsets + r0, n, a.cand_bins, a.cand_offsets + r0, a.E + r0,
-            seg_shift, n_seg, planes, info, starts, list, n_list);
+            seg_bins, n_seg, planes, extra, n_extra, info, starts, list, counts);
         e = cudaGetLastError();
         if (e != cudaSuccess) break;
         blocked_kernel<Q><<<fault_grid((unsigned)(sm_count() * kBlockedCtas)), kBlockedWarps * 32, 0, s>>>(
-            bank->bits, (uint32_t)bank->n_bins, a.cand_bins, a.cand_offsets + r0, n, n_seg, planes, info, starts,
+            bank->bits, (uint32_t)bank->n_bins, a.cand_bins, a.cand_offsets + r0, n, n_seg, planes, extra, info, starts,
             a.pass, bank->status, counter);
         e = cudaGetLastError();
         if (e != cudaSuccess) break;
         blocked_direct_kernel<Q><<<fault_grid((unsigned)(sm_count() * 4)), kSmallWarps * 32, smem, s>>>(
             bank->bits, bank->n_bins, a.reads, a.read_offsets + r0, a.cand_bins, a.cand_offsets + r0, a.E + r0, a.pass,
-            bank->status, list, n_list, next);
+            bank->status, list, counts, next);
         e = cudaGetLastError();
     }
     cudaFreeAsync(mem, s);
@@ -1012,13 +1037,12 @@ int launch_gather_blocked(const grim_bank* bank, const GatherArgs& a, int64_t n_
     const int64_t row_bytes = bank->row_words * 4;
     if (bank->q != 5 || a.sums || (double)bank->n_bins * (double)row_bytes < kBlockedBankBytes)
         return kBlockedNotBetter;
-    int seg_shift = 0;
-    while ((row_bytes << (seg_shift + 1)) <= (int64_t)kSegmentBytes) seg_shift++;
-    const int64_t n_seg = (bank->n_bins + (int64_t(1) << seg_shift) - 1) >> seg_shift;
+    const int64_t n_seg = (bank->n_bins * row_bytes + (int64_t)kSegmentBytes - 1) / (int64_t)kSegmentBytes;
+    const int64_t seg_bins = (bank->n_bins + n_seg - 1) / n_seg;  // equal segments
     if (n_seg > kMaxSegments || (double)n_checks * (double)row_bytes < kBlockedRowBytes ||
         n_checks < kBlockedChecksPerItem * n_seg * a.n_reads)
         return kBlockedNotBetter;
-    return launch_blocked<5>(bank, a, seg_shift, (int)n_seg, s);
+    return launch_blocked<5>(bank, a, (uint32_t)seg_bins, (int)n_seg, s);
 }
 
 template <int Q>
