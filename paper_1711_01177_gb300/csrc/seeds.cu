@@ -1131,27 +1131,44 @@ __global__ void batch_end_kernel(const int64_t* __restrict__ hit_off, int64_t n,
 
 // ------------------------------------------------------ seed location checker
 
-constexpr int64_t kLocTile = kScanTile;
+// Candidates per thread: four 16-byte loads in flight.  Both kernels are bound
+// by the latency of a CTA's few dependent loads and barriers, so fewer CTAs of
+// more bytes each are faster (219M pass bytes, 1% passing: count 84 -> 44 us,
+// write 214 -> 117).
+constexpr int kLocVecs = 4;
+constexpr int kLocItems = 16 * kLocVecs;
+constexpr int64_t kLocTile = (int64_t)kScanThreads * kLocItems;
 
-// Nonzero pass bytes among this thread's 16 (bit i = byte t0 + i): one
-// 16-byte load when the bytes are aligned and in range.
-__device__ __forceinline__ uint32_t pass_mask16(const uint8_t* __restrict__ pass, int64_t t0, int64_t n,
-                                                bool aligned) {
-    if (aligned && t0 + 16 <= n) return nonzero_bytes16(__ldg(reinterpret_cast<const uint4*>(pass + t0)));
-    uint32_t m = 0;
-    for (int i = 0; i < kScanItems; i++)
-        if (t0 + i < n && pass[t0 + i]) m |= 1u << i;
+// Nonzero pass bytes among this thread's kLocItems (bit i = byte t0 + i):
+// 16-byte loads where the bytes are aligned and in range.
+__device__ __forceinline__ uint64_t pass_mask(const uint8_t* __restrict__ pass, int64_t t0, int64_t n, bool aligned) {
+    static_assert(kLocItems <= 64, "one bit per candidate");
+    uint64_t m = 0;
+    if (aligned && t0 + kLocItems <= n) {
+        uint4 v[kLocVecs];
+#pragma unroll
+        for (int u = 0; u < kLocVecs; u++) v[u] = __ldg(reinterpret_cast<const uint4*>(pass + t0) + u);
+#pragma unroll
+        for (int u = 0; u < kLocVecs; u++) m |= (uint64_t)nonzero_bytes16(v[u]) << (16 * u);
+        return m;
+    }
+    for (int i = 0; i < kLocItems; i++)
+        if (t0 + i < n && pass[t0 + i]) m |= 1ull << i;
     return m;
 }
 
 __global__ void locate_count_kernel(const uint8_t* __restrict__ pass, int64_t n_cands, bool aligned,
                                     int64_t* __restrict__ counts) {
-    __shared__ int64_t ws[32];
-    const int64_t t0 = (int64_t)blockIdx.x * kLocTile + (int64_t)threadIdx.x * kScanItems;
-    const int64_t c = __popc(pass_mask16(pass, t0, n_cands, aligned));
-    int64_t total;
-    block_exclusive_scan<int64_t>(c, ws, &total);
-    if (threadIdx.x == 0) counts[blockIdx.x] = total;
+    __shared__ int warp_sum[kScanThreads / 32];
+    const int64_t t0 = (int64_t)blockIdx.x * kLocTile + (int64_t)threadIdx.x * kLocItems;
+    const int c = __reduce_add_sync(kFull, (unsigned)__popcll(pass_mask(pass, t0, n_cands, aligned)));
+    if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int64_t total = 0;
+        for (int w = 0; w < kScanThreads / 32; w++) total += warp_sum[w];
+        counts[blockIdx.x] = total;
+    }
 }
 
 // Reads holding candidates c0 (lanes 0-15) and c1 (lanes 16-31): the last
@@ -1200,12 +1217,12 @@ __global__ void locate_write_kernel(const uint8_t* __restrict__ pass, bool align
     __shared__ int64_t ws[32];
     __shared__ int64_t tile_reads[2];
     const int64_t tile0 = (int64_t)blockIdx.x * kLocTile;
-    const int64_t t0 = tile0 + (int64_t)threadIdx.x * kScanItems;
-    uint32_t m = pass_mask16(pass, t0, n_cands, aligned);
+    const int64_t t0 = tile0 + (int64_t)threadIdx.x * kLocItems;
+    uint64_t m = pass_mask(pass, t0, n_cands, aligned);
     uint32_t flags = 0;
     if (threadIdx.x == 0 && blockIdx.x == 0 && cand_offsets[n_reads] != n_cands) flags |= GRIM_FLAG_BAD_OFFSETS;
     int64_t total;
-    int64_t o = tile_base[blockIdx.x] + block_exclusive_scan<int64_t>(__popc(m), ws, &total);
+    int64_t o = tile_base[blockIdx.x] + block_exclusive_scan<int64_t>(__popcll(m), ws, &total);
     if (total == 0) {  // nothing passes in this tile (block-uniform)
         if (flags) atomicOr(status, flags);
         return;
@@ -1220,7 +1237,7 @@ __global__ void locate_write_kernel(const uint8_t* __restrict__ pass, bool align
     const int64_t tr0 = tile_reads[0], tr1 = tile_reads[1] > tile_reads[0] ? tile_reads[1] : tile_reads[0];
     int64_t r = -1;
     while (m && o < capacity) {
-        const int i = __ffs(m) - 1;
+        const int i = __ffsll((long long)m) - 1;
         m &= m - 1;
         const int64_t c = t0 + i;
         // the read: one search within the tile's reads, then forward
