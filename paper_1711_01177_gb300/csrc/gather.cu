@@ -34,6 +34,8 @@
 //   5. every lane then holds one whole sum of the window, compares it with
 //      the threshold and stores its pass byte (and sum): 32 bytes of one
 //      window land together (step 5).
+#include <type_traits>
+
 #include "grim_internal.cuh"
 #include "tokens.cuh"
 
@@ -279,7 +281,17 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
             for (int u = 0; u < G::kVPL; u++) pl[p][u] = planes[p * G::kRowVecs + s + u * G::kLPB];
     }
     static_assert(S::kWinSteps == G::kLPB, "one step of the window per lane of a row group");
-    for (int w0 = 0; w0 < n; w0 += 32) {
+    // full: all 32 rows of the window exist, so its steps are one straight piece
+    // of code whose loads, logic and shuffles interleave; the read's last rows
+    // test before each step.  Only for the folded planes that nearly every read
+    // has (SPARSE): with a second loop for every number of planes the code no
+    // longer fits the instruction cache.  Tests everywhere / straight for SPARSE /
+    // straight for all: 1M reads of 75 candidates, bank in L2, 1.490 / 1.373 /
+    // 1.524 ms; 200,000 of 1,000 2.62 / 2.25 / 2.26; q = 6, 290M checks, 16.6 /
+    // 15.9-16.1 / 15.9; 3.1 Gbp by segment 25.2 / 23.0 / 27.5, read from HBM (100,000
+    // reads) 4.12 / 3.7 / 4.13.
+    auto window = [&](auto full_window, int w0) {
+        constexpr bool full = decltype(full_window)::value;
         const uint32_t win_after = window_id(cands, w0 + 64 + lane, n);  // two windows ahead
         StepReducer<S::kWinSteps> red;
         // 16-step windows (q = 6) run as two passes of one unrolled 8-step
@@ -293,7 +305,7 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
             const int t = h * kPass + tl;
             const int c0 = w0 + t * G::kBPS;
             uint32_t part = 0;
-            if (c0 < n) {  // warp-uniform
+            if (full || c0 < n) {  // warp-uniform
                 // request the rows kAhead steps ahead (window position t + kAhead)
                 {
                     const int ahead = t + S::kAhead;
@@ -339,7 +351,7 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
         const int j = s * G::kBPS + g;
         const int c = w0 + j;
         const uint32_t id = __shfl_sync(kFull, st.win_cur, j);
-        if (c < n) {
+        if (full || c < n) {
             const bool in_range = id < n_bins32;
             if (!in_range) flags |= GRIM_FLAG_BAD_BIN;
             const uint32_t sum = in_range ? red.total : 0u;
@@ -348,7 +360,11 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
         }
         st.win_cur = st.win_next;
         st.win_next = win_after;
-    }
+    };
+    int w = 0;
+    if constexpr (SPARSE)
+        for (; w + 32 <= n; w += 32) window(std::true_type{}, w);
+    for (; w < n; w += 32) window(std::false_type{}, w);
 }
 
 // Outputs of a read whose sum is 0 for every candidate (no tokens, or a
@@ -738,11 +754,12 @@ static int launch_range(const grim_bank* bank, const GatherArgs& a, int64_t r0, 
 //      next read's planes (cp.async) and candidate ids come in while one is
 //      scored;
 //   3. blocked_direct_kernel: the listed reads as in gather_kernel.
-// 3.1 Gbp, 1M reads, 1.67e9 checks: 38.2 -> 25.3 ms, of which the ordering
-// (step 1) is 1.25.  Bound: rows from the L2 (8.8 TB/s of the 14 a sequential
-// read of it reaches).  Segments of 32 MB 29.9 (half as many candidates per
-// read and segment), of 128 MB 27.9; 3 CTAs of 8 warps 26.4; two row buffers
-// and 4 CTAs 27.3.
+// 3.1 Gbp, 1M reads, 1.67e9 checks: 38.2 -> 23.0 ms, of which the ordering
+// (step 1) is 1.25.  Bound: issue, and the breaks between the short runs of two
+// reads (rows from the L2 at 9.8 TB/s; loads that do nothing else reach 15).
+// When it took 25.3: segments of 32 MB 29.9 (half as many candidates per read
+// and segment), of 128 MB 27.9; 3 CTAs of 8 warps 26.4; two row buffers and 4
+// CTAs 27.3.
 constexpr size_t kSegmentBytes = size_t(72) << 20;
 // Where the line lies (q = 5, reads of 100 bases unless said; by segment
 // against the claiming kernel, ms): rows of 8 GB read in all - 3.1 Gbp 30,000
@@ -854,7 +871,7 @@ blocked_prep_kernel(const uint8_t* __restrict__ reads, const int64_t* __restrict
 }
 
 constexpr int kBlockedWarps = 4;
-constexpr int kBlockedCtas = 7;  // per SM (72 registers)
+constexpr int kBlockedCtas = 6;  // per SM (80 registers); 7 of 72 24.7 ms for 23.0, 5 of 96 23.6
 
 template <int Q>
 __global__ void __launch_bounds__(kBlockedWarps * 32, kBlockedCtas)
