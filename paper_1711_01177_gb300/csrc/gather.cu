@@ -323,7 +323,7 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
                 }
                 // score this step's rows
                 const uint4 (&v)[G::kVPL] = st.r[tl % S::kBufs];
-                if constexpr (NP > 0 && G::kVPL == 2) {
+                if constexpr (NP > 0 && NP <= 2 && G::kVPL == 2) {
                     part = row_sum8<NP, SPARSE>(v, pl);
                 } else if (NP > 0) {
 #pragma unroll
@@ -362,7 +362,7 @@ __device__ __forceinline__ void score_read(Stream<Q, DEEP>& st, const uint4* __r
         st.win_next = win_after;
     };
     int w = 0;
-    if constexpr (SPARSE)
+    if constexpr (SPARSE && NP == 2)
         for (; w + 32 <= n; w += 32) window(std::true_type{}, w);
     for (; w < n; w += 32) window(std::false_type{}, w);
 }
@@ -380,7 +380,7 @@ __device__ __forceinline__ void write_constant(int64_t co, int64_t ce, const uin
     }
 }
 
-// Reads with at most 255 token positions (q <= 5) count their tokens in bytes: one
+// Reads of up to 1,024 token positions (q <= 5) count their tokens in bytes: one
 // shared atomic add per token, no carries.  The counters sit in the upper
 // half of the warp's plane area (planes 8-15, which such reads never use)
 // in a transposed order: the counter of token t is byte (t / 8) % 4 of
@@ -426,11 +426,12 @@ __device__ __forceinline__ int planes_from_counters(uint32_t* __restrict__ plane
     return used;
 }
 
-// First word of a warp's plane area that must be zero between reads: its
-// upper half for q <= 5 (the byte counters; the planes proper are written
-// whole), all of it for q = 6 (planes only ever built by carries).
+// First word of a warp's plane area that must be zero between reads: all but
+// four planes for q <= 5 (the byte counters, and planes few reads have; the
+// lowest are written whole from the counters, or zeroed before a carry chain),
+// all of it for q = 6 (planes only ever built by carries).
 template <int Q>
-constexpr int kCleanFrom = Q <= 5 ? 8 * GatherGeo<Q>::kRowWords : 0;
+constexpr int kCleanFrom = Q <= 5 ? 4 * GatherGeo<Q>::kRowWords : 0;
 
 // Shared-memory set-up of a gather warp.
 template <int Q>
@@ -438,6 +439,11 @@ __device__ __forceinline__ void gather_warp_setup(uint32_t* planes, int lane) {
     for (int i = kCleanFrom<Q> + lane; i < GatherGeo<Q>::kPlaneWords; i += 32) planes[i] = 0;
     __syncwarp();
 }
+
+// Reads of up to this many tokens are counted in bytes (q <= 5), whose sum
+// tells whether one ran over (137,000 reads of 270-300 bases with few
+// candidates: 164 us by carry chains, 146 so).
+constexpr int kCountedTokens = 1024;
 
 // Steps 1-2: the count planes of a read of n_tok token positions; returns how
 // many there are.  Whole warp; bad_base collects codes > 3.
@@ -447,13 +453,21 @@ __device__ __forceinline__ int build_planes(const uint8_t* __restrict__ rd, int 
     constexpr int RW = GatherGeo<Q>::kRowWords;
     // byte counters, then the planes from them (q <= 5); for q = 6 the 4096
     // counters cost more to cut into planes than the carries they save
-    if (Q <= 5 && n_tok <= 255) {
+    if (Q <= 5 && n_tok <= kCountedTokens) {
         for_each_token5<Q>(rd, L, lane, bad_base,
                            [&](uint32_t tok) { atomicAdd(&planes[counter_word<Q>(tok)], 1u << (tok & 0x18u)); });
         __syncwarp();
-        return planes_from_counters<Q>(planes, lane);
+        bool fits = n_tok <= 255;
+        if (!fits) {  // a byte that ran over took 255 or 256 from the bytes' sum
+            uint32_t sum = 0;
+            for (int i = 8 * RW + lane; i < 16 * RW; i += 32) sum = __dp4a(planes[i], 0x01010101u, sum);
+            fits = __reduce_add_sync(kFull, sum) == (uint32_t)n_tok;
+        }
+        if (fits) return planes_from_counters<Q>(planes, lane);
+        for (int i = 8 * RW + lane; i < 16 * RW; i += 32) planes[i] = 0;
     }
-    // q = 6 and longer reads: a carry chain of atomicXor per token
+    // q = 6, longer reads and a token of more than 255 times: a carry chain of
+    // atomicXor per token
     for (int i = lane; i < kCleanFrom<Q>; i += 32) planes[i] = 0;
     __syncwarp();
     int top = -1;  // highest plane this lane set
@@ -535,7 +549,7 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
             // the read's planes: one, two or three in registers, the top one
             // folded when it is sparse enough; anything else from shared memory
             bool sparse = false;
-            if (G::kVPL == 2 && used >= 2 && used <= 3) {
+            if (G::kVPL == 2 && used == 2) {
                 const uint4* top = planes4 + (used - 1) * G::kRowVecs + lane % G::kLPB;
                 sparse = sparse_plane(top[0], top[G::kLPB * (G::kVPL - 1)]);
             }
@@ -547,8 +561,8 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
                                              flags);
             else if (used == 2)
                 score_read<Q, 2, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums_r, lane, flags);
-            else if (Q <= 5 && used == 3 && (sparse || G::kVPL == 1))  // for q = 6 three planes stay in shared memory
-                score_read<Q, 3, DEEP, G::kVPL == 2>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co,
+            else if (Q <= 5 && used == 3)  // for q = 6 three planes stay in shared memory
+                score_read<Q, 3, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co,
                                                      sums_r, lane, flags);
             else
                 score_read<Q, 0, DEEP>(st, planes4, used, T, n_c, cands, bank, n_bins32, pass + co, sums_r, lane, flags);
