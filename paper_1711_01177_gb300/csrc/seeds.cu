@@ -310,7 +310,8 @@ struct alignas(16) FastSmem {
 // The seeds of each read of the batch, 16 lanes per read: (at, end) with vote
 // i < end of the seed at location at + i, as FastSmem holds them.  Done here,
 // a read's group starts its loads of locations two dependent loads after its
-// offsets instead of four (reads with more seeds look theirs up themselves).
+// offsets instead of four (reads with more seeds, and those of small batches,
+// look theirs up themselves).
 __global__ void seed_lookup_kernel(const uint32_t* __restrict__ idx_off, int k, const uint8_t* __restrict__ reads,
                                    const int64_t* __restrict__ read_offsets, int64_t n, uint2* __restrict__ seeds) {
     const int lane = threadIdx.x & 15;
@@ -403,7 +404,7 @@ __device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP>& sm, int64_t r, co
 #pragma unroll
     for (int i = 0; i < F::kWords / 4 / T; i++)
         reinterpret_cast<uint4*>(sm.map)[i * T + t] = make_uint4(0, 0, 0, 0);
-    if (ns <= kStoredSeeds) {
+    if (seeds && ns <= kStoredSeeds) {
         if (t < kStoredSeeds) {
             const uint2 v = __ldg(seeds + r * kStoredSeeds + t);
             sm.seed_at[t] = v.x;
@@ -1113,9 +1114,11 @@ __global__ void seed_copy_kernel(const uint32_t* __restrict__ H, const int64_t* 
 
 // next batch [r0, r1): the most reads after r0 whose votes fit `budget`
 // (at least one read), at most max_reads.
-// out = {hit_off[r0], r1, hit_off[r1], hit_off[n]}.
+// out = {hit_off[r0], r1, hit_off[r1], hit_off[n]}; also empties the batch's
+// lists (n_list[0 .. 3)).
 __global__ void batch_end_kernel(const int64_t* __restrict__ hit_off, int64_t n, int64_t r0, int64_t budget,
-                                 int64_t max_reads, int64_t* __restrict__ out) {
+                                 int64_t max_reads, int64_t* __restrict__ out, uint32_t* __restrict__ n_list) {
+    n_list[0] = n_list[1] = n_list[2] = 0;
     const int64_t h0 = hit_off[r0];
     int64_t lo = r0 + 1, hi = (n - r0) < max_reads ? n : r0 + max_reads;
     while (lo < hi) {  // largest r1 in [r0 + 1, hi] with hit_off[r1] - h0 <= budget (or r0 + 1)
@@ -1410,7 +1413,7 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
     }
     for (int64_t r0 = 0; r0 < n_reads && e == cudaSuccess && rc == GRIM_OK;) {
         int64_t b[4];
-        grim::batch_end_kernel<<<grim::fault_grid(1), 1, 0, s>>>(hit_off, n_reads, r0, kBudget, kMaxReads, info);
+        grim::batch_end_kernel<<<grim::fault_grid(1), 1, 0, s>>>(hit_off, n_reads, r0, kBudget, kMaxReads, info, slow);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(b, info, sizeof(b), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1433,26 +1436,33 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         // three lists and their lengths: reads of more votes than the batch's
         // group size takes (tried again with larger groups), and the rest
         uint32_t *n_list = slow, *list0 = slow + 4, *list1 = list0 + nb, *list2 = list1 + nb;
-        e = cudaMemsetAsync(n_list, 0, 16, s);
-        if (e != cudaSuccess) break;
         // threads per read by the batch's mean votes, with room for about three
         // times it (at 1,700 votes: 256 x 16 10.0 ms a call, 128 x 24 11.1,
         // whose reads of over 3,072 votes then take the larger groups)
         const int64_t mean = votes / nb;
-        const int64_t lookup_blocks = (nb * 16 + threads - 1) / threads;
-        grim::seed_lookup_kernel<<<grim::fault_grid((unsigned)(lookup_blocks < 65535 ? lookup_blocks : 65535)),
-                                   threads, 0, s>>>(idx->offsets, idx->k, reads, read_offsets + r0, nb, seeds);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) break;
-        const grim::FastArgs fa{idx,     reads,  read_offsets + r0, seeds, nb,  hit_off + r0, h0,
-                                bin_len, n_bins, cap,               H,     kept};
-        if (mean <= 160) e = grim::launch_seed_fast<32, 16>(fa, nullptr, nullptr, list0, n_list, s);
-        else if (mean <= 400) e = grim::launch_seed_fast<64, 16>(fa, nullptr, nullptr, list0, n_list, s);
-        else if (mean <= 800) e = grim::launch_seed_fast<64, 24>(fa, nullptr, nullptr, list0, n_list, s);
-        else if (mean <= 1200) e = grim::launch_seed_fast<128, 24>(fa, nullptr, nullptr, list0, n_list, s);
-        else e = grim::launch_seed_fast<256, 16>(fa, nullptr, nullptr, list0, n_list, s);
-        if (e == cudaSuccess) e = grim::launch_seed_fast<256, 24>(fa, list0, n_list, list1, n_list + 1, s);
-        if (e == cudaSuccess) e = grim::launch_seed_fast<512, 24>(fa, list1, n_list + 1, list2, n_list + 2, s);
+        // a small batch is a chain of launches of a few us each: the seeds are
+        // looked up by the reads' groups and what these leave goes straight to the
+        // last kernels (863 reads of 2.6 Mbp: 123 -> 112 us a call)
+        const bool small = nb <= 16 * (int64_t)grim::sm_count();
+        if (!small) {
+            const int64_t lookup_blocks = (nb * 16 + threads - 1) / threads;
+            grim::seed_lookup_kernel<<<grim::fault_grid((unsigned)(lookup_blocks < 65535 ? lookup_blocks : 65535)),
+                                       threads, 0, s>>>(idx->offsets, idx->k, reads, read_offsets + r0, nb, seeds);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) break;
+        }
+        const grim::FastArgs fa{idx,     reads,  read_offsets + r0, small ? nullptr : seeds, nb,  hit_off + r0, h0,
+                                bin_len, n_bins, cap,               H,                       kept};
+        uint32_t *left = small ? list2 : list0, *n_left = small ? n_list + 2 : n_list;
+        if (mean <= 160) e = grim::launch_seed_fast<32, 16>(fa, nullptr, nullptr, left, n_left, s);
+        else if (mean <= 400) e = grim::launch_seed_fast<64, 16>(fa, nullptr, nullptr, left, n_left, s);
+        else if (mean <= 800) e = grim::launch_seed_fast<64, 24>(fa, nullptr, nullptr, left, n_left, s);
+        else if (mean <= 1200) e = grim::launch_seed_fast<128, 24>(fa, nullptr, nullptr, left, n_left, s);
+        else e = grim::launch_seed_fast<256, 16>(fa, nullptr, nullptr, left, n_left, s);
+        if (!small) {
+            if (e == cudaSuccess) e = grim::launch_seed_fast<256, 24>(fa, list0, n_list, list1, n_list + 1, s);
+            if (e == cudaSuccess) e = grim::launch_seed_fast<512, 24>(fa, list1, n_list + 1, list2, n_list + 2, s);
+        }
         if (e != cudaSuccess) break;
         const unsigned few = (unsigned)(nb < 4 * grim::sm_count() ? nb : 4 * grim::sm_count());
         grim::seed_expand_kernel<<<grim::fault_grid(few), threads, 0, s>>>(
