@@ -18,7 +18,7 @@
 //      window of Sec. 3.2 step 1);
 //   2. each token is counted in a byte counter in shared memory (one
 //      atomic add), and the count planes are cut out of the counters with
-//      masks and shifts; for q = 6 and for reads of more than 255 tokens it
+//      masks and shifts; for q = 6 and for reads of more than 1,024 tokens it
 //      is added to the bit-sliced planes by a carry chain of atomicXor;
 //   3. every lane keeps its slice of the planes in registers (reads with up
 //      to three planes, two for q = 6) or reads it from shared memory (more
