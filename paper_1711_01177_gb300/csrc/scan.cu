@@ -294,7 +294,9 @@ struct ScanParams {
 };
 
 // Appends the passing (read, bin) pairs of one group of reads: sums[i] is
-// the sum of read n0 + i for this thread's bin.  Rare path.
+// the sum of read n0 + i for this thread's bin.  Rare path.  Ends with the
+// warp converged: the lanes part where their pairs are stored, and the next
+// round's tensor-memory load needs all of them together.
 template <int NG>
 __device__ __forceinline__ void scan_emit(const ScanParams& P, const int* sums, int n0, int valid_reads,
                                           const int32_t* __restrict__ sT, const uint32_t* __restrict__ sRid,
@@ -323,6 +325,7 @@ __device__ __forceinline__ void scan_emit(const ScanParams& P, const int* sums, 
             }
         }
     }
+    __syncwarp();
 }
 
 // Epilogue of one work item for reads with D base-4 digits (N = 192 / D
