@@ -185,38 +185,94 @@ __device__ __forceinline__ uint32_t packed_word(const uint8_t* __restrict__ ref2
     return v;
 }
 
-__device__ __forceinline__ uint32_t add_cc(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm volatile("add.cc.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint32_t addc_cc(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm volatile("addc.cc.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
+// s + p over N words, low word first: s becomes the sum.  The condition code
+// lives within one asm statement; from one statement to the next the carry is
+// a value (kIn: `carry` goes in; kOut: it comes out).
+template <int N, bool kIn, bool kOut>
+__device__ __forceinline__ void add_words(uint32_t* s, const uint32_t* p, uint32_t& carry) {
+    static_assert(N == 1 || N == 2 || N == 3 || N == 8, "the group sizes below");
+#define GRIM_ADD(words, ...)                                                                               \
+    if constexpr (kIn && kOut) asm("add.cc.u32 %0, %0, 0xffffffff;\n\taddc" words "addc.u32 %0, 0, 0;" __VA_ARGS__); \
+    else if constexpr (kIn) asm("add.cc.u32 %0, %0, 0xffffffff;\n\taddc" words __VA_ARGS__);               \
+    else if constexpr (kOut) asm("add" words "addc.u32 %0, 0, 0;" __VA_ARGS__);                            \
+    else asm("add" words __VA_ARGS__)
+    if constexpr (N == 1) {
+        GRIM_ADD(".cc.u32 %1, %1, %2;\n\t", : "+r"(carry), "+r"(s[0]) : "r"(p[0]));
+    } else if constexpr (N == 2) {
+        GRIM_ADD(".cc.u32 %1, %1, %3;\n\taddc.cc.u32 %2, %2, %4;\n\t",
+                 : "+r"(carry), "+r"(s[0]), "+r"(s[1]) : "r"(p[0]), "r"(p[1]));
+    } else if constexpr (N == 3) {
+        GRIM_ADD(".cc.u32 %1, %1, %4;\n\taddc.cc.u32 %2, %2, %5;\n\taddc.cc.u32 %3, %3, %6;\n\t",
+                 : "+r"(carry), "+r"(s[0]), "+r"(s[1]), "+r"(s[2]) : "r"(p[0]), "r"(p[1]), "r"(p[2]));
+    } else {
+        GRIM_ADD(".cc.u32 %1, %1, %9;\n\taddc.cc.u32 %2, %2, %10;\n\taddc.cc.u32 %3, %3, %11;\n\t"
+                 "addc.cc.u32 %4, %4, %12;\n\taddc.cc.u32 %5, %5, %13;\n\taddc.cc.u32 %6, %6, %14;\n\t"
+                 "addc.cc.u32 %7, %7, %15;\n\taddc.cc.u32 %8, %8, %16;\n\t",
+                 : "+r"(carry), "+r"(s[0]), "+r"(s[1]), "+r"(s[2]), "+r"(s[3]), "+r"(s[4]), "+r"(s[5]), "+r"(s[6]),
+                   "+r"(s[7])
+                 : "r"(p[0]), "r"(p[1]), "r"(p[2]), "r"(p[3]), "r"(p[4]), "r"(p[5]), "r"(p[6]), "r"(p[7]));
+    }
+#undef GRIM_ADD
 }
 
-// One read base: Pv / Mv (rows whose vertical difference is +1 / -1) advance
-// by a column.  eq(w): match mask of word w.
-template <int W, typename Eq>
-__device__ __forceinline__ void rows_step(uint32_t (&Pv)[W], uint32_t (&Mv)[W], Eq&& eq) {
-    uint32_t ph_below = 0x80000000u, mh_below = 0;  // D[0][j] - D[0][j-1] = +1
+// Words of one addition at most.  Two operations a column pass the carry over
+// each boundary, which hardly shows while the GPU is full (18 words, 1M
+// locations: 2.07 ms in groups of 2 to 18); a call of few locations waits for
+// each column's chain, and what that takes turns on the order the groups give
+// the code.  500 locations, us, for groups of 2, 3, 6 and one statement a word
+// whose carry the next one took from the condition code: 15 words 57.4, 63.5,
+// 63.9, 58; 18 words 71.6, 67.6, 73.3, 67.6; 26 words -, 88, 82, 99; 32 words
+// -, 113, 103 (8: 103), 108.
+template <int W>
+constexpr int kAddWords = W == 15 ? 2 : W < 32 ? 3 : 8;
+
+// Words of the next group when `left` are still to be added: groups as equal
+// as they can be.
+template <int W>
+__host__ __device__ constexpr int add_group(int left) {
+    const int groups = (left + kAddWords<W> - 1) / kAddWords<W>;
+    return groups > 0 ? (left + groups - 1) / groups : 0;
+}
+
+// Words W0 .. W - 1 of one read base's step, a group at a time; e: the match
+// masks of the first group.  The next group's are asked for before this one is
+// worked on.
+template <int W, int W0, int N, typename Eq>
+__device__ __forceinline__ void rows_words(uint32_t (&Pv)[W], uint32_t (&Mv)[W], const uint32_t (&e)[N], Eq&& eq,
+                                           uint32_t carry, uint32_t ph_below, uint32_t mh_below) {
+    constexpr int kNext = add_group<W>(W - W0 - N);
+    uint32_t e_next[kNext > 0 ? kNext : 1], s[N];
 #pragma unroll
-    for (int w = 0; w < W; w++) {
-        const uint32_t e = eq(w), pv = Pv[w], mv = Mv[w];
-        const uint32_t a = e & pv;
-        const uint32_t s = w == 0 ? add_cc(a, pv) : addc_cc(a, pv);
-        const uint32_t xv = e | mv;
-        const uint32_t xh = (s ^ pv) | e;
+    for (int i = 0; i < kNext; i++) e_next[i] = eq(W0 + N + i);
+#pragma unroll
+    for (int i = 0; i < N; i++) s[i] = e[i] & Pv[W0 + i];
+    add_words<N, (W0 > 0), (kNext > 0)>(s, Pv + W0, carry);
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        const uint32_t pv = Pv[W0 + i], mv = Mv[W0 + i];
+        const uint32_t xv = e[i] | mv;
+        const uint32_t xh = (s[i] ^ pv) | e[i];
         const uint32_t ph = mv | ~(xh | pv);
         const uint32_t mh = pv & xh;
         const uint32_t phs = __funnelshift_l(ph_below, ph, 1);
         const uint32_t mhs = __funnelshift_l(mh_below, mh, 1);
         ph_below = ph;
         mh_below = mh;
-        Pv[w] = mhs | ~(xv | phs);
-        Mv[w] = phs & xv;
+        Pv[W0 + i] = mhs | ~(xv | phs);
+        Mv[W0 + i] = phs & xv;
     }
+    if constexpr (kNext > 0) rows_words<W, W0 + N>(Pv, Mv, e_next, eq, carry, ph_below, mh_below);
+}
+
+// One read base: Pv / Mv (rows whose vertical difference is +1 / -1) advance
+// by a column.  eq(w): match mask of word w.
+template <int W, typename Eq>
+__device__ __forceinline__ void rows_step(uint32_t (&Pv)[W], uint32_t (&Mv)[W], Eq&& eq) {
+    constexpr int kFirst = add_group<W>(W);
+    uint32_t e[kFirst];
+#pragma unroll
+    for (int i = 0; i < kFirst; i++) e[i] = eq(i);
+    rows_words<W, 0>(Pv, Mv, e, eq, 0u, 0x80000000u, 0u);  // D[0][j] - D[0][j-1] = +1
 }
 
 template <int W>
