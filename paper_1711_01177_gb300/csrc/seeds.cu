@@ -270,39 +270,45 @@ struct FastDiv {
 // 3.27 -> 2.03.  What it replaced wrote every vote to memory, read it back and
 // sorted it by buckets with 256 threads a read; the same buckets sorted by
 // insertion here, without the trip through memory, took 17.5 ms.
-constexpr int kFastSeeds = 64;    // seeds per read
+constexpr int kFewSeeds = 64;     // seeds per read, unless the group is built for more (MANY)
 constexpr int kStoredSeeds = 16;  // of which seed_lookup_kernel leaves the location ranges of the first
 constexpr int kFastExtra = 128;   // bins beside the first of their cell
 constexpr int kFastLoads = 4;     // locations in flight per thread
 constexpr int kFastHist = 64;     // the cap's vote threshold lies below this
 
 // T threads per read, each holding up to V votes in registers; CAP: reads may
-// have more bins than the cap keeps.
-template <int T, int V, bool CAP>
+// have more bins than the cap keeps; MANY: reads may have more than kFewSeeds
+// seeds (a vote's seed is then searched for, not walked to).
+template <int T, int V, bool CAP, bool MANY>
 struct FastGeo {
     static_assert(V % 8 == 0 && V <= 32, "whole 16-byte groups of ranks, one bit per vote");
     static constexpr int kVotes = V * T;
     static constexpr int kWords = V * T;             // bitmap words: V per thread
+    static constexpr int kSeeds = MANY ? kWords / 4 : kFewSeeds;
     static constexpr int kGroups = T == 32 ? 4 : 1;  // reads side by side in a CTA
     // CTAs an SM should hold (registers): as many as the shared memory allows
     static constexpr int kMinCtas = T == 32 ? 8 : T == 512 ? (V <= 16 ? 2 : 1) : (V <= 16 ? 1280 : 896) / T;
 };
 
-template <int T, int V, bool CAP>
+template <int T, int V, bool CAP, bool MANY>
 struct alignas(16) FastSmem {
-    using F = FastGeo<T, V, CAP>;
+    using F = FastGeo<T, V, CAP, MANY>;
     uint32_t map[F::kWords];                // (with a cap: then every bin, in order)
     // the first vote's bin of every set cell, in order; from the back: the
     // votes that found their bit set
     uint32_t bin[F::kVotes];
-    uint16_t rank[F::kWords];               // set cells before each bitmap word (then every bin's votes)
+    union {
+        struct {  // until the votes are read
+            uint32_t seed_at[F::kSeeds];    // vote i of the seed lies at seed_at + i
+            uint32_t seed_end[F::kSeeds];   // votes up to and with this seed
+        };
+        alignas(16) uint16_t rank[F::kWords];  // set cells before each bitmap word (then every bin's votes)
+    };
     uint32_t votes2[CAP ? F::kVotes / 2 : 4];  // with a cap: votes of bin[], two 16-bit counts a word
     uint32_t extra[kFastExtra];             // as found, then without repeats
     uint32_t sorted[kFastExtra];
     uint32_t extra_votes[CAP ? kFastExtra : 1];
     uint32_t hist[CAP ? kFastHist : 1];     // bins by votes (the last: and more)
-    uint32_t seed_at[kFastSeeds];           // vote i of the seed lies at seed_at + i
-    uint32_t seed_end[kFastSeeds];          // votes up to and with this seed
     uint32_t warp_sum[32];
     uint32_t n_set, n_extra, n_sorted;
 };
@@ -380,15 +386,15 @@ __device__ __forceinline__ uint32_t group_scan(uint32_t v, uint32_t* warp_sum, u
 // cell_mul: floor(2^32 cells / n_bins), so that bin * cell_mul >> 32 spreads
 // the bin ids evenly and in order over the bitmap.  The whole group; ends
 // with the shared memory free for another read.
-template <int T, int V, bool CAP>
-__device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP>& sm, int64_t r, const uint32_t* __restrict__ idx_off,
+template <int T, int V, bool CAP, bool MANY>
+__device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP, MANY>& sm, int64_t r, const uint32_t* __restrict__ idx_off,
                                           const uint32_t* __restrict__ idx_pos, int k,
                                           const uint8_t* __restrict__ reads,
                                           const int64_t* __restrict__ read_offsets, const uint2* __restrict__ seeds,
                                           const int64_t* __restrict__ hit_off, int64_t h0, FastDiv bin_div,
                                           uint32_t last_bin, uint32_t cell_mul, int cap, uint32_t* __restrict__ H,
                                           int64_t* __restrict__ kept) {
-    using F = FastGeo<T, V, CAP>;
+    using F = FastGeo<T, V, CAP, MANY>;
     const int t = threadIdx.x % T, lane = threadIdx.x & 31;
     const int64_t base = hit_off[r] - h0, votes = hit_off[r + 1] - hit_off[r];
     if (votes <= 0) {
@@ -397,7 +403,7 @@ __device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP>& sm, int64_t r, co
     }
     const int64_t ro = read_offsets[r];
     const int64_t ns = n_seeds_of(read_offsets[r + 1] - ro, k);
-    if (votes > F::kVotes || ns > kFastSeeds) return false;
+    if (votes > F::kVotes || ns > F::kSeeds) return false;
     const int n = (int)votes;
 
     // the seeds' location ranges (first warp), an empty bitmap
@@ -409,6 +415,20 @@ __device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP>& sm, int64_t r, co
             const uint2 v = __ldg(seeds + r * kStoredSeeds + t);
             sm.seed_at[t] = v.x;
             sm.seed_end[t] = v.y;
+        }
+    } else if constexpr (MANY) {
+        static_assert(F::kSeeds % T == 0, "whole rounds of the group");
+        uint32_t before = 0;
+        for (int g = 0; g < (int)ns; g += T) {
+            uint32_t at = 0, m = 0, key, total;
+            if (g + t < ns && seed_key(reads + ro + (int64_t)(g + t) * k, k, &key)) {
+                at = idx_off[key];
+                m = idx_off[key + 1] - at;
+            }
+            const uint32_t o = before + group_scan<T>(m, sm.warp_sum, &total);
+            sm.seed_at[g + t] = at - o;
+            sm.seed_end[g + t] = o + m;
+            before += total;
         }
     } else if (t < 32) {
         uint32_t before = 0;
@@ -445,9 +465,23 @@ __device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP>& sm, int64_t r, co
         for (int u = 0; u < kFastLoads; u++) {
             const int i = (u0 + u) * T + t;
             if (i < n) {
-                while ((uint32_t)i >= end) {  // i < n = the last seed's end
-                    at = sm.seed_at[++sd];
-                    end = sm.seed_end[sd];
+                if constexpr (MANY) {
+                    if ((uint32_t)i >= end) {  // the first seed that ends after i
+                        int hi = (int)ns - 1;
+                        sd++;
+                        while (sd < hi) {
+                            const int mid = (sd + hi) >> 1;
+                            if ((uint32_t)i < sm.seed_end[mid]) hi = mid;
+                            else sd = mid + 1;
+                        }
+                        at = sm.seed_at[sd];
+                        end = sm.seed_end[sd];
+                    }
+                } else {
+                    while ((uint32_t)i >= end) {  // i < n = the last seed's end
+                        at = sm.seed_at[++sd];
+                        end = sm.seed_end[sd];
+                    }
                 }
                 bin[u0 + u] = __ldg(idx_pos + (at + (uint32_t)i));
                 off[u] = (uint32_t)(sd * k);
@@ -700,8 +734,8 @@ __device__ __forceinline__ bool fast_read(FastSmem<T, V, CAP>& sm, int64_t r, co
 // Every read of the batch (list == null) or the listed ones, a group of T
 // threads each; those that fast_read does not take are appended to
 // slow[0 .. *n_slow).
-template <int T, int V, bool CAP>
-__global__ void __launch_bounds__(T * FastGeo<T, V, CAP>::kGroups, FastGeo<T, V, CAP>::kMinCtas)
+template <int T, int V, bool CAP, bool MANY>
+__global__ void __launch_bounds__(T * FastGeo<T, V, CAP, MANY>::kGroups, FastGeo<T, V, CAP, MANY>::kMinCtas)
 seed_fast_kernel(const uint32_t* __restrict__ idx_off, const uint32_t* __restrict__ idx_pos, int k,
                  const uint8_t* __restrict__ reads, const int64_t* __restrict__ read_offsets,
                  const uint2* __restrict__ seeds, int64_t n_reads, const uint32_t* __restrict__ list,
@@ -709,14 +743,14 @@ seed_fast_kernel(const uint32_t* __restrict__ idx_off, const uint32_t* __restric
                  FastDiv bin_div, uint32_t last_bin,
                  uint32_t cell_mul, int cap, uint32_t* __restrict__ H, int64_t* __restrict__ kept,
                  uint32_t* __restrict__ slow, uint32_t* __restrict__ n_slow) {
-    using F = FastGeo<T, V, CAP>;
+    using F = FastGeo<T, V, CAP, MANY>;
     extern __shared__ __align__(16) uint8_t fast_smem_raw[];
     const int group = threadIdx.x / T;
-    FastSmem<T, V, CAP>& sm = reinterpret_cast<FastSmem<T, V, CAP>*>(fast_smem_raw)[group];
+    FastSmem<T, V, CAP, MANY>& sm = reinterpret_cast<FastSmem<T, V, CAP, MANY>*>(fast_smem_raw)[group];
     const int64_t n = list ? (int64_t)*n_list : n_reads;
     for (int64_t i = (int64_t)blockIdx.x * F::kGroups + group; i < n; i += (int64_t)gridDim.x * F::kGroups) {
         const int64_t r = list ? (int64_t)list[i] : i;
-        const bool taken = fast_read<T, V, CAP>(sm, r, idx_off, idx_pos, k, reads, read_offsets, seeds, hit_off, h0,
+        const bool taken = fast_read<T, V, CAP, MANY>(sm, r, idx_off, idx_pos, k, reads, read_offsets, seeds, hit_off, h0,
                                         bin_div, last_bin, cell_mul, cap, H, kept);
         if (!taken && threadIdx.x % T == 0) slow[atomicAdd(n_slow, 1u)] = (uint32_t)r;
         group_sync<T>();
@@ -724,8 +758,10 @@ seed_fast_kernel(const uint32_t* __restrict__ idx_off, const uint32_t* __restric
 }
 
 // The votes of the listed reads list[0 .. *n_list) of the batch: read r's
-// bins at H[hit_off[r] - h0 ...], one CTA per read, its warps taking the seeds
-// in turn (a listed read has thousands of locations per seed).
+// bins at H[hit_off[r] - h0 ...].  A short list is of reads with thousands of
+// locations per seed: one CTA per read, its warps taking the seeds in turn.  A
+// long one (reads of thousands of seeds of few locations) gives each read as
+// many of its warps as there are to go round.
 __global__ void seed_expand_kernel(const uint32_t* __restrict__ idx_off, const uint32_t* __restrict__ idx_pos, int k,
                                    const uint8_t* __restrict__ reads, const int64_t* __restrict__ read_offsets,
                                    const uint32_t* __restrict__ list, const uint32_t* __restrict__ n_list,
@@ -733,7 +769,10 @@ __global__ void seed_expand_kernel(const uint32_t* __restrict__ idx_off, const u
                                    uint32_t last_bin, uint32_t* __restrict__ H) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int64_t n = *n_list;
-    for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
+    int team = warps;  // warps per read: 1, 2, 4 or 8
+    while (team > 1 && n * team > (int64_t)gridDim.x * warps) team >>= 1;
+    const int64_t stride = (int64_t)gridDim.x * warps / team;
+    for (int64_t i = ((int64_t)blockIdx.x * warps + warp) / team; i < n; i += stride) {
         const int64_t r = list[i];
         const int64_t ro = read_offsets[r], L = read_offsets[r + 1] - ro;
         const int64_t ns = n_seeds_of(L, k);
@@ -752,7 +791,7 @@ __global__ void seed_expand_kernel(const uint32_t* __restrict__ idx_off, const u
                 if (lane >= o) x += y;
             }
             const int cnt = ns - g < 32 ? (int)(ns - g) : 32;
-            for (int sd = warp; sd < cnt; sd += warps) {
+            for (int sd = warp % team; sd < cnt; sd += team) {
                 const uint32_t sa = __shfl_sync(kFull, a, sd), sm = __shfl_sync(kFull, m, sd);
                 const int64_t to = w + __shfl_sync(kFull, x, sd) - sm;
                 const uint32_t o = (uint32_t)((g + sd) * k);
@@ -1058,15 +1097,15 @@ struct FastArgs {
     int64_t* kept;
 };
 
-template <int T, int V, bool CAP>
+template <int T, int V, bool CAP, bool MANY>
 cudaError_t launch_fast(const FastArgs& a, const uint32_t* list, const uint32_t* n_list, uint32_t* slow,
                         uint32_t* n_slow, cudaStream_t s) {
-    using F = FastGeo<T, V, CAP>;
-    constexpr size_t smem = sizeof(FastSmem<T, V, CAP>) * F::kGroups;
+    using F = FastGeo<T, V, CAP, MANY>;
+    constexpr size_t smem = sizeof(FastSmem<T, V, CAP, MANY>) * F::kGroups;
     static DeviceCache attr[64];  // per device
     const int dev = a.idx->device;
     if (smem > 48 * 1024 && dev >= 0 && dev < 64 && !attr[dev].load()) {
-        const cudaError_t e = cudaFuncSetAttribute(seed_fast_kernel<T, V, CAP>,
+        const cudaError_t e = cudaFuncSetAttribute(seed_fast_kernel<T, V, CAP, MANY>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr[dev].store(1);
@@ -1074,7 +1113,7 @@ cudaError_t launch_fast(const FastArgs& a, const uint32_t* list, const uint32_t*
     const uint64_t mul = ((uint64_t)(32 * F::kWords) << 32) / (uint64_t)a.n_bins;
     int64_t blocks = (a.nb + F::kGroups - 1) / F::kGroups;
     if (list && blocks > 4 * sm_count()) blocks = 4 * sm_count();  // few, taken in turn
-    seed_fast_kernel<T, V, CAP><<<grim::fault_grid((unsigned)blocks), T * F::kGroups, smem, s>>>(
+    seed_fast_kernel<T, V, CAP, MANY><<<grim::fault_grid((unsigned)blocks), T * F::kGroups, smem, s>>>(
         a.idx->offsets, a.idx->positions, a.idx->k, a.reads, a.read_offsets, a.seeds, a.nb, list, n_list, a.hit_off, a.h0,
         FastDiv((uint32_t)a.bin_len), (uint32_t)(a.n_bins - 1),
         (uint32_t)(mul < 0xFFFFFFFFull ? mul : 0xFFFFFFFFull), a.cap, a.H, a.kept, slow, n_slow);
@@ -1082,11 +1121,11 @@ cudaError_t launch_fast(const FastArgs& a, const uint32_t* list, const uint32_t*
 }
 
 // A cap that no read the kernel takes can exceed needs no votes per bin.
-template <int T, int V>
+template <int T, int V, bool MANY = false>
 cudaError_t launch_seed_fast(const FastArgs& a, const uint32_t* list, const uint32_t* n_list, uint32_t* slow,
                              uint32_t* n_slow, cudaStream_t s) {
-    return a.cap >= FastGeo<T, V, true>::kVotes ? launch_fast<T, V, false>(a, list, n_list, slow, n_slow, s)
-                                                : launch_fast<T, V, true>(a, list, n_list, slow, n_slow, s);
+    return a.cap >= FastGeo<T, V, true, MANY>::kVotes ? launch_fast<T, V, false, MANY>(a, list, n_list, slow, n_slow, s)
+                                                : launch_fast<T, V, true, MANY>(a, list, n_list, slow, n_slow, s);
 }
 
 // cand_bins[cand_off[r] ...] <- the kept bins of read r (warp per read),
@@ -1114,10 +1153,11 @@ __global__ void seed_copy_kernel(const uint32_t* __restrict__ H, const int64_t* 
 
 // next batch [r0, r1): the most reads after r0 whose votes fit `budget`
 // (at least one read), at most max_reads.
-// out = {hit_off[r0], r1, hit_off[r1], hit_off[n]}; also empties the batch's
-// lists (n_list[0 .. 3)).
-__global__ void batch_end_kernel(const int64_t* __restrict__ hit_off, int64_t n, int64_t r0, int64_t budget,
-                                 int64_t max_reads, int64_t* __restrict__ out, uint32_t* __restrict__ n_list) {
+// out = {hit_off[r0], r1, hit_off[r1], hit_off[n], bases of the batch}; also
+// empties the batch's lists (n_list[0 .. 3)).
+__global__ void batch_end_kernel(const int64_t* __restrict__ hit_off, const int64_t* __restrict__ read_offsets,
+                                 int64_t n, int64_t r0, int64_t budget, int64_t max_reads, int64_t* __restrict__ out,
+                                 uint32_t* __restrict__ n_list) {
     n_list[0] = n_list[1] = n_list[2] = 0;
     const int64_t h0 = hit_off[r0];
     int64_t lo = r0 + 1, hi = (n - r0) < max_reads ? n : r0 + max_reads;
@@ -1130,6 +1170,7 @@ __global__ void batch_end_kernel(const int64_t* __restrict__ hit_off, int64_t n,
     out[1] = lo;
     out[2] = hit_off[lo];
     out[3] = hit_off[n];
+    out[4] = read_offsets[lo] - read_offsets[r0];
 }
 
 // ------------------------------------------------------ seed location checker
@@ -1412,8 +1453,9 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         }
     }
     for (int64_t r0 = 0; r0 < n_reads && e == cudaSuccess && rc == GRIM_OK;) {
-        int64_t b[4];
-        grim::batch_end_kernel<<<grim::fault_grid(1), 1, 0, s>>>(hit_off, n_reads, r0, kBudget, kMaxReads, info, slow);
+        int64_t b[5];
+        grim::batch_end_kernel<<<grim::fault_grid(1), 1, 0, s>>>(hit_off, read_offsets, n_reads, r0, kBudget, kMaxReads,
+                                                                 info, slow);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(b, info, sizeof(b), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1454,18 +1496,27 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         const grim::FastArgs fa{idx,     reads,  read_offsets + r0, small ? nullptr : seeds, nb,  hit_off + r0, h0,
                                 bin_len, n_bins, cap,               H,                       kept};
         uint32_t *left = small ? list2 : list0, *n_left = small ? n_list + 2 : n_list;
-        if (mean <= 160) e = grim::launch_seed_fast<32, 16>(fa, nullptr, nullptr, left, n_left, s);
+        // most reads of more seeds than the groups below take (those of 769 bases
+        // and more at k = 12)
+        const int64_t mean_seeds = b[4] / nb / idx->k;
+        if (mean_seeds > grim::kFewSeeds * 3 / 4) {
+            if (mean <= 800 && mean_seeds <= 300)
+                e = grim::launch_seed_fast<64, 24, true>(fa, nullptr, nullptr, left, n_left, s);
+            else
+                e = grim::launch_seed_fast<256, 24, true>(fa, nullptr, nullptr, left, n_left, s);
+        } else if (mean <= 160) e = grim::launch_seed_fast<32, 16>(fa, nullptr, nullptr, left, n_left, s);
         else if (mean <= 400) e = grim::launch_seed_fast<64, 16>(fa, nullptr, nullptr, left, n_left, s);
         else if (mean <= 800) e = grim::launch_seed_fast<64, 24>(fa, nullptr, nullptr, left, n_left, s);
         else if (mean <= 1200) e = grim::launch_seed_fast<128, 24>(fa, nullptr, nullptr, left, n_left, s);
         else e = grim::launch_seed_fast<256, 16>(fa, nullptr, nullptr, left, n_left, s);
         if (!small) {
-            if (e == cudaSuccess) e = grim::launch_seed_fast<256, 24>(fa, list0, n_list, list1, n_list + 1, s);
-            if (e == cudaSuccess) e = grim::launch_seed_fast<512, 24>(fa, list1, n_list + 1, list2, n_list + 2, s);
+            if (e == cudaSuccess) e = grim::launch_seed_fast<256, 24, true>(fa, list0, n_list, list1, n_list + 1, s);
+            if (e == cudaSuccess) e = grim::launch_seed_fast<512, 24, true>(fa, list1, n_list + 1, list2, n_list + 2, s);
         }
         if (e != cudaSuccess) break;
         const unsigned few = (unsigned)(nb < 4 * grim::sm_count() ? nb : 4 * grim::sm_count());
-        grim::seed_expand_kernel<<<grim::fault_grid(few), threads, 0, s>>>(
+        const int64_t all = 8 * (int64_t)grim::sm_count();  // CTAs the GPU holds
+        grim::seed_expand_kernel<<<grim::fault_grid((unsigned)(nb < all ? nb : all)), threads, 0, s>>>(
                 idx->offsets, idx->positions, idx->k, reads, read_offsets + r0, list2, n_list + 2, hit_off + r0, h0,
                 (uint32_t)bin_len, (uint32_t)(n_bins - 1), H);
         grim::seed_dedupe_kernel<<<grim::fault_grid(few), grim::kDedupThreads, grim::kDedupSmemBytes, s>>>(
