@@ -1128,6 +1128,16 @@ cudaError_t launch_seed_fast(const FastArgs& a, const uint32_t* list, const uint
                                                 : launch_fast<T, V, true, MANY>(a, list, n_list, slow, n_slow, s);
 }
 
+// The reads that a first kernel left to list0 by the larger groups; what these
+// leave: list2.  n_list: the three lists' lengths.
+template <bool MANY>
+cudaError_t launch_larger(const FastArgs& a, uint32_t* list0, uint32_t* list1, uint32_t* list2, uint32_t* n_list,
+                          cudaStream_t s) {
+    const cudaError_t e = launch_seed_fast<256, 24, MANY>(a, list0, n_list, list1, n_list + 1, s);
+    if (e != cudaSuccess) return e;
+    return launch_seed_fast<512, 24, MANY>(a, list1, n_list + 1, list2, n_list + 2, s);
+}
+
 // cand_bins[cand_off[r] ...] <- the kept bins of read r (warp per read),
 // entries at or beyond `capacity` dropped.
 __global__ void seed_copy_kernel(const uint32_t* __restrict__ H, const int64_t* __restrict__ hit_off, int64_t h0,
@@ -1496,10 +1506,13 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         const grim::FastArgs fa{idx,     reads,  read_offsets + r0, small ? nullptr : seeds, nb,  hit_off + r0, h0,
                                 bin_len, n_bins, cap,               H,                       kept};
         uint32_t *left = small ? list2 : list0, *n_left = small ? n_list + 2 : n_list;
-        // most reads of more seeds than the groups below take (those of 769 bases
-        // and more at k = 12)
+        // batches with reads of more seeds than most groups take (769 bases and more
+        // at k = 12), by their mean length: the groups for many seeds cost the others
+        // a search per vote (20,000 reads of 300 bases on 3.1 Gbp, 25 seeds: 2.73 ms
+        // for 2.58)
         const int64_t mean_seeds = b[4] / nb / idx->k;
-        if (mean_seeds > grim::kFewSeeds * 3 / 4) {
+        const bool many = mean_seeds > grim::kFewSeeds / 2;
+        if (many) {
             if (mean <= 800 && mean_seeds <= 300)
                 e = grim::launch_seed_fast<64, 24, true>(fa, nullptr, nullptr, left, n_left, s);
             else
@@ -1509,10 +1522,9 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         else if (mean <= 800) e = grim::launch_seed_fast<64, 24>(fa, nullptr, nullptr, left, n_left, s);
         else if (mean <= 1200) e = grim::launch_seed_fast<128, 24>(fa, nullptr, nullptr, left, n_left, s);
         else e = grim::launch_seed_fast<256, 16>(fa, nullptr, nullptr, left, n_left, s);
-        if (!small) {
-            if (e == cudaSuccess) e = grim::launch_seed_fast<256, 24, true>(fa, list0, n_list, list1, n_list + 1, s);
-            if (e == cudaSuccess) e = grim::launch_seed_fast<512, 24, true>(fa, list1, n_list + 1, list2, n_list + 2, s);
-        }
+        if (!small && e == cudaSuccess)
+            e = many ? grim::launch_larger<true>(fa, list0, list1, list2, n_list, s)
+                     : grim::launch_larger<false>(fa, list0, list1, list2, n_list, s);
         if (e != cudaSuccess) break;
         const unsigned few = (unsigned)(nb < 4 * grim::sm_count() ? nb : 4 * grim::sm_count());
         const int64_t all = 8 * (int64_t)grim::sm_count();  // CTAs the GPU holds
