@@ -1494,8 +1494,11 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         const int64_t mean = votes / nb;
         // a small batch is a chain of launches of a few us each: the seeds are
         // looked up by the reads' groups and what these leave goes straight to the
-        // last kernels (863 reads of 2.6 Mbp: 123 -> 112 us a call)
-        const bool small = nb <= 16 * (int64_t)grim::sm_count();
+        // last kernels (863 reads of 2.6 Mbp: 123 -> 112 us a call).  Only while
+        // these leave next to none: the last kernels are slow (2,000 reads of 300
+        // bases on 3.1 Gbp, 5,000 votes each: 1,231 us that way, 577 by the larger
+        // groups; 1,000 of 100, 1,700 votes each: 213 and 175).
+        const bool small = nb <= 16 * (int64_t)grim::sm_count() && mean <= 800;
         if (!small) {
             const int64_t lookup_blocks = (nb * 16 + threads - 1) / threads;
             grim::seed_lookup_kernel<<<grim::fault_grid((unsigned)(lookup_blocks < 65535 ? lookup_blocks : 65535)),
