@@ -274,6 +274,7 @@ constexpr int kFewSeeds = 64;     // seeds per read, unless the group is built f
 constexpr int kStoredSeeds = 16;  // of which seed_lookup_kernel leaves the location ranges of the first
 constexpr int kFastExtra = 128;   // bins beside the first of their cell
 constexpr int kFastLoads = 4;     // locations in flight per thread
+constexpr int kSmallSeedReads = 32;  // reads per SM of a small batch, at most
 constexpr int kFastHist = 64;     // the cap's vote threshold lies below this
 
 // T threads per read, each holding up to V votes in registers; CAP: reads may
@@ -1128,11 +1129,12 @@ cudaError_t launch_seed_fast(const FastArgs& a, const uint32_t* list, const uint
                                                 : launch_fast<T, V, true, MANY>(a, list, n_list, slow, n_slow, s);
 }
 
-// The reads that a first kernel left to list0 by the larger groups; what these
-// leave: list2.  n_list: the three lists' lengths.
+// The reads that a first kernel left to list0 by the larger groups, by both or
+// by the largest alone; what these leave: list2.  n_list: the lists' lengths.
 template <bool MANY>
-cudaError_t launch_larger(const FastArgs& a, uint32_t* list0, uint32_t* list1, uint32_t* list2, uint32_t* n_list,
-                          cudaStream_t s) {
+cudaError_t launch_larger(const FastArgs& a, bool both, uint32_t* list0, uint32_t* list1, uint32_t* list2,
+                          uint32_t* n_list, cudaStream_t s) {
+    if (!both) return launch_seed_fast<512, 24, MANY>(a, list0, n_list, list2, n_list + 2, s);
     const cudaError_t e = launch_seed_fast<256, 24, MANY>(a, list0, n_list, list1, n_list + 1, s);
     if (e != cudaSuccess) return e;
     return launch_seed_fast<512, 24, MANY>(a, list1, n_list + 1, list2, n_list + 2, s);
@@ -1164,11 +1166,13 @@ __global__ void seed_copy_kernel(const uint32_t* __restrict__ H, const int64_t* 
 // next batch [r0, r1): the most reads after r0 whose votes fit `budget`
 // (at least one read), at most max_reads.
 // out = {hit_off[r0], r1, hit_off[r1], hit_off[n], bases of the batch}; also
-// empties the batch's lists (n_list[0 .. 3)).
+// empties the batch's lists (n_list[0 .. 3)) and starts the first batch's
+// candidate offsets.
 __global__ void batch_end_kernel(const int64_t* __restrict__ hit_off, const int64_t* __restrict__ read_offsets,
                                  int64_t n, int64_t r0, int64_t budget, int64_t max_reads, int64_t* __restrict__ out,
-                                 uint32_t* __restrict__ n_list) {
+                                 uint32_t* __restrict__ n_list, int64_t* __restrict__ cand_off) {
     n_list[0] = n_list[1] = n_list[2] = 0;
+    if (r0 == 0) cand_off[0] = 0;
     const int64_t h0 = hit_off[r0];
     int64_t lo = r0 + 1, hi = (n - r0) < max_reads ? n : r0 + max_reads;
     while (lo < hi) {  // largest r1 in [r0 + 1, hi] with hit_off[r1] - h0 <= budget (or r0 + 1)
@@ -1421,10 +1425,21 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
     const int threads = 256;
     const int64_t warp_blocks = (n_reads * 32 + threads - 1) / threads;
     const unsigned blocks = (unsigned)(warp_blocks < 65535 ? warp_blocks : 65535);
-    int64_t* hit_off = nullptr;
+    const int64_t kBudget = int64_t(1) << 28;     // votes per batch
+    const int64_t kMaxReads = int64_t(1) << 20;   // reads per batch
+    // the call's fixed working memory, in one piece: every allocation and its
+    // release costs a short call 1-2 us
+    const int64_t max_nb = n_reads < kMaxReads ? n_reads : kMaxReads;
+    const int64_t small_reads = grim::kSmallSeedReads * (int64_t)grim::sm_count();
+    const size_t seeds_bytes = n_reads > small_reads ? (size_t)max_nb * grim::kStoredSeeds * sizeof(uint2) : 0;
     int64_t* info = nullptr;  // batch bounds
-    GRIM_CUDA_TRY(grim::scratch_alloc((void**)&hit_off, (size_t)(n_reads + 1) * 8, s));
-    GRIM_CUDA_TRY(grim::scratch_alloc((void**)&info, 64, s));  // batch bounds
+    GRIM_CUDA_TRY(grim::scratch_alloc(
+        (void**)&info, 64 + seeds_bytes + (size_t)(n_reads + 1 + max_nb) * 8 + (size_t)(3 * max_nb + 4) * 4, s));
+    // location ranges of the batch's seeds
+    uint2* seeds = seeds_bytes ? reinterpret_cast<uint2*>(info + 8) : nullptr;
+    int64_t* hit_off = info + 8 + seeds_bytes / 8;
+    int64_t* kept = hit_off + n_reads + 1;
+    uint32_t* slow = reinterpret_cast<uint32_t*>(kept + max_nb);  // lists of the reads the fast path leaves
     int rc = GRIM_OK;
     grim::seed_hits_kernel<<<grim::fault_grid(blocks), threads, 0, s>>>(
             idx->offsets, idx->k, reads, read_offsets, n_reads, hit_off);
@@ -1441,31 +1456,15 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
                                            (int)grim::kDedupSmemBytes));
         smem_set[dev].store(1);
     }
-    const int64_t kBudget = int64_t(1) << 28;     // votes per batch
-    const int64_t kMaxReads = int64_t(1) << 20;   // reads per batch
     // scratch kept across batches (freeing it would hand it back to the
     // pool at every synchronisation): votes as u32 (H) and 2 u32 per vote (S)
     uint32_t* H = nullptr;
     unsigned long long* S = nullptr;
-    int64_t* kept = nullptr;
-    uint2* seeds = nullptr;    // location ranges of the batch's seeds
-    uint32_t* slow = nullptr;  // lists of the reads the fast path leaves
     int64_t cap_votes = 0;
-    if (e == cudaSuccess && rc == GRIM_OK) {
-        const int64_t max_nb = n_reads < kMaxReads ? n_reads : kMaxReads;
-        e = grim::scratch_alloc((void**)&kept, (size_t)max_nb * 8, s);
-        if (e == cudaSuccess)
-            e = grim::scratch_alloc((void**)&seeds, (size_t)max_nb * grim::kStoredSeeds * sizeof(uint2), s);
-        if (e == cudaSuccess) e = grim::scratch_alloc((void**)&slow, (size_t)(3 * max_nb + 4) * 4, s);
-        if (e == cudaSuccess) {
-            grim::set_value_kernel<int64_t><<<grim::fault_grid(1), 1, 0, s>>>(cand_offsets, 0, nullptr);
-            e = cudaGetLastError();
-        }
-    }
     for (int64_t r0 = 0; r0 < n_reads && e == cudaSuccess && rc == GRIM_OK;) {
         int64_t b[5];
         grim::batch_end_kernel<<<grim::fault_grid(1), 1, 0, s>>>(hit_off, read_offsets, n_reads, r0, kBudget, kMaxReads,
-                                                                 info, slow);
+                                                                 info, slow, cand_offsets);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(b, info, sizeof(b), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1490,23 +1489,26 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         uint32_t *n_list = slow, *list0 = slow + 4, *list1 = list0 + nb, *list2 = list1 + nb;
         // threads per read by the batch's mean votes, with room for about three
         // times it (at 1,700 votes: 256 x 16 10.0 ms a call, 128 x 24 11.1,
-        // whose reads of over 3,072 votes then take the larger groups)
+        // whose reads of over 3,072 votes then take the larger groups); a small
+        // batch does not fill the GPU, and a larger group has its read sooner
+        // (1,000 reads on 1 Gbp, 540 votes: 137 us by 64 x 24, 118 by 256 x 16)
         const int64_t mean = votes / nb;
         // a small batch is a chain of launches of a few us each: the seeds are
         // looked up by the reads' groups and what these leave goes straight to the
-        // last kernels (863 reads of 2.6 Mbp: 123 -> 112 us a call).  Only while
-        // these leave next to none: the last kernels are slow (2,000 reads of 300
-        // bases on 3.1 Gbp, 5,000 votes each: 1,231 us that way, 577 by the larger
-        // groups; 1,000 of 100, 1,700 votes each: 213 and 175).
-        const bool small = nb <= 16 * (int64_t)grim::sm_count() && mean <= 800;
-        if (!small) {
+        // last kernels (800 reads of 2.6 Mbp: 120 -> 101 us a call; 2,500 of 20 Mbp
+        // 122 -> 110; 4,000 of 400 Mbp 147 -> 131).  Only while these leave next to
+        // none: the last kernels are slow (2,000 reads of 300 bases on 3.1 Gbp, 5,000
+        // votes each: 1,231 us that way, 590 by the larger groups; 1,000 of 100, 1,700
+        // votes each: 213 and 150).
+        const bool small = nb <= small_reads && mean <= 800;
+        if (!small && seeds) {
             const int64_t lookup_blocks = (nb * 16 + threads - 1) / threads;
             grim::seed_lookup_kernel<<<grim::fault_grid((unsigned)(lookup_blocks < 65535 ? lookup_blocks : 65535)),
                                        threads, 0, s>>>(idx->offsets, idx->k, reads, read_offsets + r0, nb, seeds);
             e = cudaGetLastError();
             if (e != cudaSuccess) break;
         }
-        const grim::FastArgs fa{idx,     reads,  read_offsets + r0, small ? nullptr : seeds, nb,  hit_off + r0, h0,
+        const grim::FastArgs fa{idx,     reads,  read_offsets + r0, small ? nullptr : seeds, nb, hit_off + r0, h0,
                                 bin_len, n_bins, cap,               H,                       kept};
         uint32_t *left = small ? list2 : list0, *n_left = small ? n_list + 2 : n_list;
         // batches with reads of more seeds than most groups take (769 bases and more
@@ -1520,14 +1522,21 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
                 e = grim::launch_seed_fast<64, 24, true>(fa, nullptr, nullptr, left, n_left, s);
             else
                 e = grim::launch_seed_fast<256, 24, true>(fa, nullptr, nullptr, left, n_left, s);
-        } else if (mean <= 160) e = grim::launch_seed_fast<32, 16>(fa, nullptr, nullptr, left, n_left, s);
+        } else if (small && mean > 500) e = grim::launch_seed_fast<256, 16>(fa, nullptr, nullptr, left, n_left, s);
+        else if (mean <= 160) e = grim::launch_seed_fast<32, 16>(fa, nullptr, nullptr, left, n_left, s);
         else if (mean <= 400) e = grim::launch_seed_fast<64, 16>(fa, nullptr, nullptr, left, n_left, s);
         else if (mean <= 800) e = grim::launch_seed_fast<64, 24>(fa, nullptr, nullptr, left, n_left, s);
         else if (mean <= 1200) e = grim::launch_seed_fast<128, 24>(fa, nullptr, nullptr, left, n_left, s);
         else e = grim::launch_seed_fast<256, 16>(fa, nullptr, nullptr, left, n_left, s);
-        if (!small && e == cudaSuccess)
-            e = many ? grim::launch_larger<true>(fa, list0, list1, list2, n_list, s)
-                     : grim::launch_larger<false>(fa, list0, list1, list2, n_list, s);
+        if (!small && e == cudaSuccess) {
+            // both larger groups where the list is long enough for the smaller one to
+            // pay (a launch with a few reads takes 10-18 us: 2,500 reads on 3.1 Gbp
+            // 229 us by both, 204 by the largest alone; 5,000 303 and 280; 40,000 on
+            // 1 Gbp 453 either way; 2,000 of 5,000 votes each 587 and 600)
+            const bool both = nb > 200 * (int64_t)grim::sm_count() || mean > 2000;
+            e = many ? grim::launch_larger<true>(fa, both, list0, list1, list2, n_list, s)
+                     : grim::launch_larger<false>(fa, both, list0, list1, list2, n_list, s);
+        }
         if (e != cudaSuccess) break;
         const unsigned few = (unsigned)(nb < 4 * grim::sm_count() ? nb : 4 * grim::sm_count());
         const int64_t all = 8 * (int64_t)grim::sm_count();  // CTAs the GPU holds
@@ -1551,11 +1560,7 @@ int grim_seed_candidates(const grim_seed_index* idx, const uint8_t* reads, const
         e = cudaMemcpyAsync(&total, cand_offsets + n_reads, 8, cudaMemcpyDeviceToHost, s);
     if (H) cudaFreeAsync(H, s);
     if (S) cudaFreeAsync(S, s);
-    if (kept) cudaFreeAsync(kept, s);
-    if (slow) cudaFreeAsync(slow, s);
-    if (seeds) cudaFreeAsync(seeds, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(hit_off, s);
     cudaFreeAsync(info, s);
     if (e != cudaSuccess) {
         grim::set_last_cuda_error(e);
