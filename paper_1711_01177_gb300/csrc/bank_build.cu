@@ -23,8 +23,9 @@
 // q = 6 and geometry the main kernel does not take: bank_build_tile_kernel,
 // the same P and R rows for a run of cores per CTA, row-major.
 //
-// Fallback kernel (bins or overlaps too long for either): one CTA owns a run
-// of consecutive bins and keeps their rows in shared memory; its threads walk
+// Short bins with long overlaps, whose rows are ORs of many others that hold
+// few bits (and bins or overlaps too long for either): one CTA owns a run of
+// consecutive bins and keeps their rows in shared memory; its threads walk
 // every token start of the run's spans once and set the token's bit in every
 // bin of the run whose span holds it with a shared-memory atomicOr; the rows
 // then leave in 16-byte stores.
@@ -34,7 +35,8 @@ namespace grim {
 
 constexpr int kBuildThreads = 256;
 constexpr int kBuildSmemBytes = 16384;    // bin rows per CTA
-constexpr int kTileStageBytes = 16384;    // staged packed reference per CTA
+constexpr int kBuildStageBytes = 32768;   // staged packed reference per CTA
+constexpr int kTileStageBytes = 16384;    // the same of the tile kernel
 
 template <int Q>
 __global__ void __launch_bounds__(kBuildThreads)
@@ -76,6 +78,92 @@ bank_build_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bin_len,
     }
     __syncthreads();
 
+    uint4* dst = reinterpret_cast<uint4*>(bank + b0 * G::kRowWords);
+    for (int i = threadIdx.x; i < nb * row4; i += blockDim.x) dst[i] = smem4[i];
+}
+
+// The same with the run's packed reference bytes staged in shared memory,
+// and each thread rolls the token through a contiguous stretch of token
+// starts (two instructions per base) while tracking, without divisions, the
+// first and last bin whose span holds the current token.
+template <int Q>
+__global__ void __launch_bounds__(kBuildThreads)
+bank_build_staged_kernel(const uint8_t* __restrict__ ref2bit, int64_t len, int bin_len, int overlap, int64_t n_bins,
+                         int bins_per_cta, uint32_t* __restrict__ bank) {
+    using G = Geo<Q>;
+    constexpr uint32_t kMask = (Q == 16) ? 0xffffffffu : ((1u << (2 * Q)) - 1u);
+    extern __shared__ uint4 smem4[];
+    uint32_t* sbits = reinterpret_cast<uint32_t*>(smem4);
+    const int64_t b0 = (int64_t)blockIdx.x * bins_per_cta;
+    const int nb = (int)((n_bins - b0) < bins_per_cta ? (n_bins - b0) : bins_per_cta);
+    const int row4 = G::kRowWords / 4;
+    uint32_t* sref = sbits + (size_t)bins_per_cta * G::kRowWords;  // packed reference, 16 bases per word
+
+    const int64_t p0 = b0 * (int64_t)bin_len;
+    int64_t pend = (b0 + nb) * (int64_t)bin_len + overlap;
+    if (pend > len) pend = len;
+    // packed bytes [4*word0, 4*ceil(pend/16)) of the reference, as words
+    const int64_t word0 = p0 >> 4;
+    const int64_t byte_end = (pend + 3) >> 2;
+    const int nwords = (int)(((pend + 15) >> 4) - word0);
+    for (int i = threadIdx.x; i < nb * row4; i += blockDim.x) smem4[i] = make_uint4(0, 0, 0, 0);
+    for (int i = threadIdx.x; i < nwords; i += blockDim.x) {
+        uint32_t v = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int64_t byte = 4 * (word0 + i) + k;
+            if (byte < byte_end) v |= (uint32_t)__ldg(ref2bit + byte) << (8 * k);
+        }
+        sref[i] = v;
+    }
+    __syncthreads();
+
+    // token starts i in [p0, pend - Q], split into one stretch per thread
+    const int n_starts = (int)(pend - Q + 1 - p0);
+    if (n_starts > 0) {
+        const int per = (n_starts + blockDim.x - 1) / blockDim.x;
+        const int s0 = threadIdx.x * per;
+        const int s1 = min(n_starts, s0 + per);
+        if (s0 < s1) {
+            // bases stream from a one-word buffer: x = position - 16*word0
+            int x = (int)(p0 + s0 - 16 * word0);
+            uint32_t buf = sref[x >> 4] >> (2 * (x & 15));
+            int left = 16 - (x & 15);
+            auto next_base = [&]() -> uint32_t {
+                if (left == 0) {
+                    buf = sref[x >> 4];
+                    left = 16;
+                }
+                const uint32_t b = buf & 3u;
+                buf >>= 2;
+                --left;
+                ++x;
+                return b;
+            };
+            uint32_t tok = 0;
+#pragma unroll
+            for (int k = 0; k < Q - 1; k++) tok = (tok << 2) | next_base();
+            // bin bookkeeping for the first start, then incremental
+            const int64_t i_first = p0 + s0;
+            int64_t bhi = i_first / bin_len;                           // last bin with b*bin_len <= i
+            int64_t next_hi = (bhi + 1) * (int64_t)bin_len;           // i at which bhi grows
+            const int64_t need = i_first + Q - (int64_t)bin_len - overlap;
+            int64_t blo = need <= 0 ? 0 : (need + bin_len - 1) / bin_len;  // first bin with i+Q <= its span end
+            int64_t next_lo = blo * (int64_t)bin_len + bin_len + overlap - Q + 1;  // i at which blo grows
+            const int64_t b_last = b0 + nb - 1;
+            for (int rel = s0; rel < s1; rel++) {
+                const int64_t i = p0 + rel;
+                if (i == next_hi) { ++bhi; next_hi += bin_len; }
+                if (i == next_lo) { ++blo; next_lo += bin_len; }
+                tok = ((tok << 2) | next_base()) & kMask;
+                const uint32_t w = tok >> 5, m = 1u << (tok & 31);
+                const int lo = (int)((blo > b0 ? blo : b0) - b0);
+                const int hi = (int)((bhi < b_last ? bhi : b_last) - b0);
+                for (int b = lo; b <= hi; b++) atomicOr(&sbits[b * G::kRowWords + w], m);
+            }
+        }
+    }
+    __syncthreads();
     uint4* dst = reinterpret_cast<uint4*>(bank + b0 * G::kRowWords);
     for (int i = threadIdx.x; i < nb * row4; i += blockDim.x) dst[i] = smem4[i];
 }
@@ -502,24 +590,52 @@ static int launch_q(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s) {
     const int r_pref = e >= 0 ? (int)(e % bl) : bl;
     const int starts = e >= 0 ? bl : (bl + e > 0 ? (int)(bl + e) : 0);
     if constexpr (Q <= 5) {
-        if (bl >= kLaneMinBinLen && bl <= kLaneMaxBinLen && J <= kLaneMaxJ && ((uintptr_t)ref2bit & 3) == 0)
+        // q = 5, lengths that are no multiple of 16: a warp's 32 cores take 110 + 11 J +
+        // bl for the 31 - J rows they finish, the walk below 50 a row, 0.75 a bit and 3 a
+        // start of its core (20 Mbp, us, lanes / walk, or the tile where its rule takes
+        // them: 17 + 30 76 / 51 (tile), 17 + 250 256 / 147, 33 + 500 157 / 88 (tile),
+        // 24 + 100 66 / 68, 40 + 600 116 / 141; q = 4, 17 + 250 76 / 133)
+        const bool short_bins = Q == 5 && bl % 16 != 0 &&
+                                128 * (110 + 11 * J + bl) > (200 + 3 * (bl + (int64_t)bank->overlap) + 12 * bl) * (31 - J);
+        if (bl >= kLaneMinBinLen && bl <= kLaneMaxBinLen && J <= kLaneMaxJ && !short_bins &&
+            ((uintptr_t)ref2bit & 3) == 0)
             return bl % 16 == 0 ? launch_lanes<Q, true>(ref2bit, bank, s, starts, r_pref, (int)J)
                                 : launch_lanes<Q, false>(ref2bit, bank, s, starts, r_pref, (int)J);
     }
     // a tile of cores, as many as 16 KB of rows and 16 KB of staged bases
-    // allow, at least half of whose rows are finished
+    // allow.  It ORs 2 J + 3 rows into each row it finishes, 16 bytes at a time;
+    // the walk of a run's token starts sets bl + overlap bits a row, and passes bl
+    // starts.  What these take, in hundredths of a vector ORed (q = 6: the tile
+    // has fewer rows to spread its set-up over), from 20 Mbp banks, tile / walk, us:
+    // q = 5, 8 + 30 117 / 92, 12 + 30 72 / 78, 12 + 60 94 / 84, 15 + 30 51 / 70,
+    // 15 + 100 94 / 88, 8 + 100 264 / 135; q = 4, 8 + 100 75 / 109; q = 3, 43 /
+    // 121; q = 6, 8 + 100 989 / 246, 32 + 100 103 / 94, 64 + 900 158 / 141, 100 +
+    // 1,500 115 / 149.
     const int64_t fit = (kTileStageBytes / 4 - 4) * 16 / bl;
     const int64_t cores = fit < TileGeo<Q>::kMaxCores ? fit : TileGeo<Q>::kMaxCores;
-    if (cores > 0 && 2 * (J + 1) <= cores)
+    const int64_t finished = cores - J - 1;  // rows of a tile
+    constexpr int64_t kPerVec = Q >= 6 ? 72 : 100, kPerRow = Q >= 6 ? 2000 : 0;
+    if (cores > 0 && 2 * (J + 1) <= cores &&
+        kPerVec * (2 * J + 3) * TileGeo<Q>::kVecs * cores + kPerRow * finished <=
+            (70 * (bl + (int64_t)bank->overlap) + 275 * (int64_t)bl) * finished)
         return launch_tile<Q>(
             ref2bit, bank, s, starts, r_pref, (int)J, (int)cores,
             (size_t)(2 * cores + 1) * G::kRowWords * 4 + 4 * (size_t)((cores * bl + 30) / 16 + 2));
     const int bins_per_cta = kBuildSmemBytes / (G::kRowWords * 4);
     const int64_t blocks = (bank->n_bins + bins_per_cta - 1) / bins_per_cta;
     if (blocks > 0x7fffffff) return GRIM_ENOTSUP;
-    bank_build_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads,
-                           (size_t)bins_per_cta * G::kRowWords * 4, s>>>(
-        ref2bit, bank->len, bank->bin_len, bank->overlap, bank->n_bins, bins_per_cta, bank->bits);
+    const size_t smem_rows = (size_t)bins_per_cta * G::kRowWords * 4;
+    // staged where a run's packed reference bytes fit beside its rows
+    const int64_t stage = 4 * (((int64_t)bins_per_cta * bl + bank->overlap) / 16 + 3);
+    if (stage <= kBuildStageBytes) {
+        static_assert(kBuildSmemBytes + kBuildStageBytes <= 48 * 1024, "no attribute needed");
+        bank_build_staged_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads,
+                                      smem_rows + (size_t)((stage + 15) & ~15LL), s>>>(
+            ref2bit, bank->len, bl, bank->overlap, bank->n_bins, bins_per_cta, bank->bits);
+    } else {
+        bank_build_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads, smem_rows, s>>>(
+            ref2bit, bank->len, bl, bank->overlap, bank->n_bins, bins_per_cta, bank->bits);
+    }
     GRIM_CUDA_TRY(cudaGetLastError());
     return GRIM_OK;
 }
