@@ -427,13 +427,16 @@ static int launch_lanes(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s,
     const int out_w = 32 - (J + 1);
     const int64_t n_units = (bank->n_bins + out_w - 1) / out_w;
     const size_t smem = lane_smem_bytes<Q>(bank->bin_len);
-    static DeviceCache attr[64];  // per device: the largest size set so far
+    // per device, and the same limit whatever the bin length: of two threads in
+    // their first call neither may lower the other's
+    static DeviceCache attr[64];
     const int slot = device_slot();
     if (slot < 0) return GRIM_ENOTSUP;
-    if (attr[slot].load() < (int)smem) {
-        GRIM_CUDA_TRY(
-            cudaFuncSetAttribute(bank_build_lanes_kernel<Q, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr[slot].store((int)smem);
+    if (!attr[slot].load()) {
+        GRIM_CUDA_TRY(cudaFuncSetAttribute(bank_build_lanes_kernel<Q, WORDS>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)lane_smem_bytes<Q>(kLaneMaxBinLen)));
+        attr[slot].store(1);
     }
     int per_sm = 0;
     GRIM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bank_build_lanes_kernel<Q, WORDS>, kLaneCores, smem));
@@ -468,6 +471,7 @@ struct TileGeo {
     static constexpr int kRW = Geo<Q>::kRowWords;
     static constexpr int kMaxCores = 16384 / (4 * kRW);  // 16 KB per row set
     static constexpr int kVecs = kRW / 4;
+    static constexpr size_t kMaxSmem = (size_t)(2 * kMaxCores + 1) * kRW * 4 + kTileStageBytes;
     // byte offset of a token's row word, as a mask on the token shifted right by 3
     static constexpr uint32_t kWordMask = Q >= 3 ? (uint32_t)((1u << (2 * Q - 5)) - 1u) << 2 : 0u;
 };
@@ -565,13 +569,13 @@ static int launch_tile(const uint8_t* ref2bit, grim_bank* bank, cudaStream_t s, 
                        int cores, size_t smem) {
     const int64_t blocks = (bank->n_bins + cores - J - 2) / (cores - J - 1);
     if (blocks > 0x7fffffff) return GRIM_ENOTSUP;
-    static DeviceCache attr[64];  // per device: the largest size set so far
+    static DeviceCache attr[64];  // per device, one limit for every geometry (see launch_lanes)
     const int slot = device_slot();
     if (slot < 0) return GRIM_ENOTSUP;
-    if (smem > 48 * 1024 && attr[slot].load() < (int)smem) {
-        GRIM_CUDA_TRY(
-            cudaFuncSetAttribute(bank_build_tile_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr[slot].store((int)smem);
+    if (!attr[slot].load()) {
+        GRIM_CUDA_TRY(cudaFuncSetAttribute(bank_build_tile_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)TileGeo<Q>::kMaxSmem));
+        attr[slot].store(1);
     }
     bank_build_tile_kernel<Q><<<grim::fault_grid((unsigned)blocks), kBuildThreads, smem, s>>>(
         ref2bit, bank->len, bank->bin_len, starts, r_pref, J, cores, bank->n_bins, bank->bits);
