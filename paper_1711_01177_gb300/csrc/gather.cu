@@ -550,9 +550,10 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
             // folded when it is sparse enough; anything else from shared memory
             // q = 6: a read of one plane and a short list goes the way of two, the second
             // empty (the area is clean past `used`): short and long reads side by side
-            // then share one loop's code.  150,000 reads of 50-300 bases, 8 candidates
+            // then share one loop's code (not where a warp has one read only: 2-4%
+            // slower so).  150,000 reads of 50-300 bases, 8 candidates
             // each, 228 -> 203 us (32: 362 -> 331); long lists are faster by one plane.
-            if (Q >= 6 && used == 1 && n_c <= 96) used = 2;
+            if (Q >= 6 && !DEEP && used == 1 && n_c <= 96) used = 2;
             bool sparse = false;
             if (G::kVPL == 2 && used == 2) {
                 const uint4* top = planes4 + (used - 1) * G::kRowVecs + lane % G::kLPB;
