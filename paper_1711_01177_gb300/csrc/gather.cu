@@ -85,15 +85,16 @@ __device__ __forceinline__ void csa(uint32_t& hi, uint32_t& lo, uint32_t a, uint
 //    a bit in it (`kSparse`, checked once per read by sparse_plane), their
 //    ANDed words are simply ORed together - one three-input op per word -
 //    and counted once per vector.
-// kSparse: the top plane NP - 1 >= 1 is folded that way.
+// kSparse: the upper of two planes is folded that way.
 // 1M reads of 150 bases, 75 candidates each, bank in L2: 1.55 -> 1.49 ms;
 // 200,000 reads of 1,000 candidates 3.20 -> 2.78; q = 6, 290M checks, 18.2 ->
 // 16.6 (there the bank is read from HBM, and the adders were in use before).
 template <int NP, bool kSparse>
 __device__ __forceinline__ uint32_t row_sum8(const uint4 (&v)[2], const uint4 (&p)[NP][2]) {
+    static_assert(NP == 2 || (NP == 1 && !kSparse), "one or two planes");
     uint32_t sum = 0;
     if constexpr (kSparse) {
-        const uint4(&t)[2] = p[NP - 1];
+        const uint4(&t)[2] = p[1];
         uint32_t o0 = v[0].x & t[0].x, o1 = v[1].x & t[1].x;
         o0 |= v[0].y & t[0].y;
         o1 |= v[1].y & t[1].y;
@@ -101,7 +102,7 @@ __device__ __forceinline__ uint32_t row_sum8(const uint4 (&v)[2], const uint4 (&
         o1 |= v[1].z & t[1].z;
         o0 |= v[0].w & t[0].w;
         o1 |= v[1].w & t[1].w;
-        sum = (__popc(o0) + __popc(o1)) << (NP - 1);
+        sum = 2 * (__popc(o0) + __popc(o1));
     }
     const uint32_t a0 = v[0].x & p[0][0].x, a1 = v[0].y & p[0][0].y, a2 = v[0].z & p[0][0].z,
                    a3 = v[0].w & p[0][0].w, a4 = v[1].x & p[0][1].x, a5 = v[1].y & p[0][1].y,
@@ -112,10 +113,9 @@ __device__ __forceinline__ uint32_t row_sum8(const uint4 (&v)[2], const uint4 (&
     csa(c3, s3, s1, s2, a6);
     csa(d1, s4, c1, c2, c3);
     sum += __popc(s3) + __popc(a7);
-    if constexpr (NP - (kSparse ? 1 : 0) == 1) {
+    if constexpr (NP == 1 || kSparse) {
         return sum + 2 * __popc(s4) + 4 * __popc(d1);
     } else {
-        static_assert(NP - (kSparse ? 1 : 0) == 2, "two dense planes at most");
         const uint32_t b0 = v[0].x & p[1][0].x, b1 = v[0].y & p[1][0].y, b2 = v[0].z & p[1][0].z,
                        b3 = v[0].w & p[1][0].w, b4 = v[1].x & p[1][1].x, b5 = v[1].y & p[1][1].y,
                        b6 = v[1].z & p[1][1].z, b7 = v[1].w & p[1][1].w;
@@ -546,7 +546,7 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
         if (bad_read || used == 0)
             write_constant(co, ce, cand_bins, n_bins, !bad_read && T <= 0, pass, sums, lane, flags);
         else {
-            // the read's planes: one, two or three in registers, the top one
+            // the read's planes: one, two or three in registers, the upper of two
             // folded when it is sparse enough; anything else from shared memory
             // q = 6: a read of one plane and a short list goes the way of two, the second
             // empty (the area is clean past `used`): short and long reads side by side
@@ -556,7 +556,7 @@ __device__ __forceinline__ void gather_read(int64_t ro, int64_t re, int64_t co, 
             if (Q >= 6 && !DEEP && used == 1 && n_c <= 96) used = 2;
             bool sparse = false;
             if (G::kVPL == 2 && used == 2) {
-                const uint4* top = planes4 + (used - 1) * G::kRowVecs + lane % G::kLPB;
+                const uint4* top = planes4 + G::kRowVecs + lane % G::kLPB;
                 sparse = sparse_plane(top[0], top[G::kLPB * (G::kVPL - 1)]);
             }
             uint16_t* sums_r = sums ? sums + co : nullptr;
