@@ -24,6 +24,8 @@
 //   - grim_locate: tile counts of passing bytes -> prefix sum -> ordered
 //     write of (read, bin, span); optional segment bases copied out of the
 //     2-bit reference (one warp per segment).
+#include <type_traits>
+
 #include "grim_internal.cuh"
 
 struct grim_seed_index {
@@ -1189,37 +1191,61 @@ __global__ void batch_end_kernel(const int64_t* __restrict__ hit_off, const int6
 
 // ------------------------------------------------------ seed location checker
 
-// Candidates per thread: four 16-byte loads in flight.  Both kernels are bound
-// by the latency of a CTA's few dependent loads and barriers, so fewer CTAs of
-// more bytes each are faster (219M pass bytes, 1% passing: count 84 -> 44 us,
-// write 214 -> 117).
-constexpr int kLocVecs = 4;
-constexpr int kLocItems = 16 * kLocVecs;
-constexpr int64_t kLocTile = (int64_t)kScanThreads * kLocItems;
+// Candidates per thread: 16 (VECS = 1) while the tiles of these fill the GPU
+// once at most, else 64, four 16-byte loads in flight: both kernels are bound by
+// the latency of a CTA's few dependent loads and barriers, so fewer CTAs of more
+// bytes each are faster once there are enough (us a call, 1% passing, by 16 / by
+// 64: 1,000 bytes 25 / 29, 3M 31 / 32, 10M 44 / 35, 200M 366 / 188).
+template <int VECS>
+struct LocGeo {
+    static_assert(VECS == 1 || VECS == 4, "one bit per candidate of a thread");
+    using Mask = typename std::conditional<VECS == 1, uint32_t, uint64_t>::type;
+    static constexpr int kItems = 16 * VECS;
+    static constexpr int kTile = kScanThreads * kItems;
+    // A tile with more passing candidates than this is written in VECS rounds of 16
+    // candidates a thread: a thread that writes its own 64 leaves a warp's stores
+    // four times as far apart (200M bytes, us at once / in
+    // rounds: 5% passing 295 / 310, 8% 449 / 430, 30% 2,757 / 1,248).
+    static constexpr int kDense = VECS == 1 ? kTile : kTile / 16;
+};
 
-// Nonzero pass bytes among this thread's kLocItems (bit i = byte t0 + i):
-// 16-byte loads where the bytes are aligned and in range.
-__device__ __forceinline__ uint64_t pass_mask(const uint8_t* __restrict__ pass, int64_t t0, int64_t n, bool aligned) {
-    static_assert(kLocItems <= 64, "one bit per candidate");
-    uint64_t m = 0;
-    if (aligned && t0 + kLocItems <= n) {
-        uint4 v[kLocVecs];
+// Nonzero pass bytes among this thread's (bit i = byte t0 + i), by 16-byte
+// loads from the 16-byte boundary at or before the first of them (`shift` bytes
+// before it) where these lie among the n bytes: the masks are shifted into
+// place, not the bytes.
+template <int VECS>
+__device__ __forceinline__ typename LocGeo<VECS>::Mask pass_mask(const uint8_t* __restrict__ pass, int64_t t0, int64_t n,
+                                                                 int shift) {
+    using Mask = typename LocGeo<VECS>::Mask;
+    constexpr int kItems = LocGeo<VECS>::kItems;
+    Mask m = 0;
+    const int64_t a0 = t0 - shift;
+    if (a0 >= 0 && a0 + kItems + (shift ? 16 : 0) <= n) {
+        const uint4* p = reinterpret_cast<const uint4*>(pass + a0);
+        uint4 v[VECS];
 #pragma unroll
-        for (int u = 0; u < kLocVecs; u++) v[u] = __ldg(reinterpret_cast<const uint4*>(pass + t0) + u);
+        for (int u = 0; u < VECS; u++) v[u] = __ldg(p + u);
+        Mask above = 0;
+        if (shift) above = nonzero_bytes16(__ldg(p + VECS));  // the same for the whole call
 #pragma unroll
-        for (int u = 0; u < kLocVecs; u++) m |= (uint64_t)nonzero_bytes16(v[u]) << (16 * u);
+        for (int u = 0; u < VECS; u++) m |= (Mask)nonzero_bytes16(v[u]) << (16 * u);
+        if (shift) {
+            m = (m >> shift) | (above << (kItems - shift));
+            if (VECS == 1) m &= 0xFFFFu;
+        }
         return m;
     }
-    for (int i = 0; i < kLocItems; i++)
-        if (t0 + i < n && pass[t0 + i]) m |= 1ull << i;
+    for (int i = 0; i < kItems; i++)
+        if (t0 + i < n && pass[t0 + i]) m |= (Mask)1 << i;
     return m;
 }
 
-__global__ void locate_count_kernel(const uint8_t* __restrict__ pass, int64_t n_cands, bool aligned,
+template <int VECS>
+__global__ void locate_count_kernel(const uint8_t* __restrict__ pass, int64_t n_cands, int shift,
                                     int64_t* __restrict__ counts) {
     __shared__ int warp_sum[kScanThreads / 32];
-    const int64_t t0 = (int64_t)blockIdx.x * kLocTile + (int64_t)threadIdx.x * kLocItems;
-    const int c = __reduce_add_sync(kFull, (unsigned)__popcll(pass_mask(pass, t0, n_cands, aligned)));
+    const int64_t t0 = (int64_t)blockIdx.x * LocGeo<VECS>::kTile + (int64_t)threadIdx.x * LocGeo<VECS>::kItems;
+    const int c = __reduce_add_sync(kFull, (unsigned)__popcll(pass_mask<VECS>(pass, t0, n_cands, shift)));
     if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = c;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1265,55 +1291,75 @@ __device__ __forceinline__ int64_t read_of(const int64_t* __restrict__ co, int64
     return lo;
 }
 
-__global__ void locate_write_kernel(const uint8_t* __restrict__ pass, bool aligned,
-                                    const uint32_t* __restrict__ cand_bins, const int64_t* __restrict__ cand_offsets,
-                                    int64_t n_reads, int64_t n_cands, const int64_t* __restrict__ tile_base,
-                                    int64_t len, int64_t n_bins, int bin_len, int overlap, int64_t capacity,
-                                    uint32_t* __restrict__ loc_read, uint32_t* __restrict__ loc_bin,
-                                    int64_t* __restrict__ loc_begin, int64_t* __restrict__ loc_end,
-                                    uint32_t* __restrict__ status) {
+template <int VECS>
+__global__ void __launch_bounds__(kScanThreads)
+locate_write_kernel(const uint8_t* __restrict__ pass, int shift, const uint32_t* __restrict__ cand_bins,
+                    const int64_t* __restrict__ cand_offsets, int64_t n_reads, int64_t n_cands,
+                    const int64_t* __restrict__ tile_base, int64_t len, int64_t n_bins, int bin_len, int overlap,
+                    int64_t capacity, uint32_t* __restrict__ loc_read, uint32_t* __restrict__ loc_bin,
+                    int64_t* __restrict__ loc_begin, int64_t* __restrict__ loc_end, uint32_t* __restrict__ status) {
+    using G = LocGeo<VECS>;
     __shared__ int64_t ws[32];
     __shared__ int64_t tile_reads[2];
-    const int64_t tile0 = (int64_t)blockIdx.x * kLocTile;
-    const int64_t t0 = tile0 + (int64_t)threadIdx.x * kLocItems;
-    uint64_t m = pass_mask(pass, t0, n_cands, aligned);
+    const int64_t tile0 = (int64_t)blockIdx.x * G::kTile;
+    const int64_t t0 = tile0 + (int64_t)threadIdx.x * G::kItems;
+    typename G::Mask m = pass_mask<VECS>(pass, t0, n_cands, shift);
     uint32_t flags = 0;
     if (threadIdx.x == 0 && blockIdx.x == 0 && cand_offsets[n_reads] != n_cands) flags |= GRIM_FLAG_BAD_OFFSETS;
     int64_t total;
-    int64_t o = tile_base[blockIdx.x] + block_exclusive_scan<int64_t>(__popcll(m), ws, &total);
+    int64_t base = tile_base[blockIdx.x];
+    int64_t o = base + block_exclusive_scan<int64_t>(__popcll(m), ws, &total);
     if (total == 0) {  // nothing passes in this tile (block-uniform)
         if (flags) atomicOr(status, flags);
         return;
     }
     if (threadIdx.x < 32) {  // the reads of the tile's first and last candidates
-        const int64_t last = (tile0 + kLocTile < n_cands ? tile0 + kLocTile : n_cands) - 1;
+        const int64_t last = (tile0 + G::kTile < n_cands ? tile0 + G::kTile : n_cands) - 1;
         const int64_t rr = reads_of_half_warps(cand_offsets, n_reads, tile0, last, threadIdx.x);
         if (threadIdx.x == 0) tile_reads[0] = rr;
         if (threadIdx.x == 16) tile_reads[1] = rr;
     }
     __syncthreads();
     const int64_t tr0 = tile_reads[0], tr1 = tile_reads[1] > tile_reads[0] ? tile_reads[1] : tile_reads[0];
-    int64_t r = -1;
-    while (m && o < capacity) {
-        const int i = __ffsll((long long)m) - 1;
-        m &= m - 1;
-        const int64_t c = t0 + i;
-        // the read: one search within the tile's reads, then forward
-        if (r < 0) r = read_of(cand_offsets, tr0, tr1, c);
-        while (r + 1 < n_reads && cand_offsets[r + 1] <= c) r++;
-        const uint32_t b = cand_bins[c];
-        int64_t begin = 0, end = 0;
-        if ((int64_t)b < n_bins) {
-            begin = (int64_t)b * bin_len;
-            end = begin + bin_len + overlap < len ? begin + bin_len + overlap : len;
-        } else {
-            flags |= GRIM_FLAG_BAD_BIN;
+    const bool dense = VECS > 1 && total > G::kDense;  // block-uniform
+    __shared__ uint64_t masks[VECS > 1 ? kScanThreads : 1];
+    if (dense) {
+        masks[threadIdx.x] = m;
+        __syncthreads();
+    }
+    for (int round = 0; round < (dense ? VECS : 1); round++) {
+        int64_t c0 = t0;
+        if (dense) {  // 16 candidates, tile0 + 16 * place on
+            const int place = round * kScanThreads + threadIdx.x;
+            m = (typename G::Mask)((masks[place / VECS] >> (16 * (place % VECS))) & 0xFFFFu);
+            c0 = tile0 + 16 * place;
+            int64_t in_round;
+            const int64_t before = block_exclusive_scan<int64_t>(__popcll(m), ws, &in_round);
+            o = base + before;
+            base += in_round;
         }
-        loc_read[o] = (uint32_t)r;
-        loc_bin[o] = b;
-        if (loc_begin) loc_begin[o] = begin;
-        if (loc_end) loc_end[o] = end;
-        o++;
+        int64_t r = -1;
+        while (m && o < capacity) {
+            const int i = __ffsll((long long)m) - 1;
+            m &= m - 1;
+            const int64_t c = c0 + i;
+            // the read: one search within the tile's reads, then forward
+            if (r < 0) r = read_of(cand_offsets, tr0, tr1, c);
+            while (r + 1 < n_reads && cand_offsets[r + 1] <= c) r++;
+            const uint32_t b = cand_bins[c];
+            int64_t begin = 0, end = 0;
+            if ((int64_t)b < n_bins) {
+                begin = (int64_t)b * bin_len;
+                end = begin + bin_len + overlap < len ? begin + bin_len + overlap : len;
+            } else {
+                flags |= GRIM_FLAG_BAD_BIN;
+            }
+            loc_read[o] = (uint32_t)r;
+            loc_bin[o] = b;
+            if (loc_begin) loc_begin[o] = begin;
+            if (loc_end) loc_end[o] = end;
+            o++;
+        }
     }
     if (flags) atomicOr(status, flags);
 }
@@ -1588,19 +1634,24 @@ int grim_locate(const grim_bank* bank, const uint8_t* ref2bit, const uint32_t* c
     if (rc != GRIM_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     if (n_cands == 0) return grim::exclusive_scan<int64_t>(nullptr, n_loc, 0, 0, s);
-    const int64_t tiles = (n_cands + grim::kLocTile - 1) / grim::kLocTile;
+    // tiles of 16 candidates a thread where these fill the GPU once at most
+    const bool small = n_cands <= 8 * (int64_t)grim::sm_count() * grim::LocGeo<1>::kTile;
+    const int64_t tile = small ? grim::LocGeo<1>::kTile : grim::LocGeo<4>::kTile;
+    const int64_t tiles = (n_cands + tile - 1) / tile;
     int64_t* counts = nullptr;
     GRIM_CUDA_TRY(grim::scratch_alloc((void**)&counts, (size_t)(tiles + 1) * 8, s));
-    const bool aligned = ((uintptr_t)pass & 15) == 0;
-    grim::locate_count_kernel<<<grim::fault_grid((unsigned)tiles), grim::kScanThreads, 0, s>>>(
-            pass, n_cands, aligned, counts);
+    const int shift = (int)((uintptr_t)pass & 15);
+    const unsigned blocks = grim::fault_grid((unsigned)tiles);
+    if (small) grim::locate_count_kernel<1><<<blocks, grim::kScanThreads, 0, s>>>(pass, n_cands, shift, counts);
+    else grim::locate_count_kernel<4><<<blocks, grim::kScanThreads, 0, s>>>(pass, n_cands, shift, counts);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) rc = grim::exclusive_scan<int64_t>(counts, counts, tiles, 0, s);
     if (e == cudaSuccess && rc == GRIM_OK)
         e = cudaMemcpyAsync(n_loc, counts + tiles, 8, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess && rc == GRIM_OK) {
-        grim::locate_write_kernel<<<grim::fault_grid((unsigned)tiles), grim::kScanThreads, 0, s>>>(
-            pass, aligned, cand_bins, cand_offsets, n_reads, n_cands, counts, bank->len, bank->n_bins, bank->bin_len,
+        auto write = small ? grim::locate_write_kernel<1> : grim::locate_write_kernel<4>;
+        write<<<grim::fault_grid((unsigned)tiles), grim::kScanThreads, 0, s>>>(
+            pass, shift, cand_bins, cand_offsets, n_reads, n_cands, counts, bank->len, bank->n_bins, bank->bin_len,
             bank->overlap, capacity, loc_read, loc_bin, loc_begin, loc_end, bank->status);
         e = cudaGetLastError();
     }
