@@ -1205,7 +1205,7 @@ struct LocGeo {
     // A tile with more passing candidates than this is written in VECS rounds of 16
     // candidates a thread: a thread that writes its own 64 leaves a warp's stores
     // four times as far apart (200M bytes, us at once / in
-    // rounds: 5% passing 295 / 310, 8% 449 / 430, 30% 2,757 / 1,248).
+    // rounds: 8% passing 449 / 430, 30% 2,757 / 1,248).
     static constexpr int kDense = VECS == 1 ? kTile : kTile / 16;
 };
 
