@@ -294,9 +294,8 @@ struct ScanParams {
 };
 
 // Appends the passing (read, bin) pairs of one group of reads: sums[i] is
-// the sum of read n0 + i for this thread's bin.  Rare path.  Ends with the
-// warp converged: the lanes part where their pairs are stored, and the next
-// round's tensor-memory load needs all of them together.
+// the sum of read n0 + i for this thread's bin.  Rare path.  The lanes may part
+// where their pairs are stored.
 template <int NG>
 __device__ __forceinline__ void scan_emit(const ScanParams& P, const int* sums, int n0, int valid_reads,
                                           const int32_t* __restrict__ sT, const uint32_t* __restrict__ sRid,
@@ -325,7 +324,6 @@ __device__ __forceinline__ void scan_emit(const ScanParams& P, const int* sums, 
             }
         }
     }
-    __syncwarp();
 }
 
 // Epilogue of one work item for reads with D base-4 digits (N = 192 / D
@@ -358,6 +356,9 @@ __device__ __forceinline__ void scan_epilogue(const ScanParams& P, uint32_t tmem
             constexpr int kFirst = decltype(first_c)::value, G = NW - kFirst < GR ? NW - kFirst : GR;
             const int n0 = share * NW + kFirst;  // first read of this round
             uint32_t v[D * G];
+            // the loads need the whole warp, whose lanes the last round's emission may
+            // have parted (at the end of the emission, the barrier cost the scan 1%)
+            __syncwarp();
 #pragma unroll
             for (int d = 0; d < D; d++) tmem_ld_cols<G>(col0 + d * N + n0, v + d * G);
             tmem_wait_ld();
