@@ -59,17 +59,17 @@ SUMMARY_KEY = {"plain": "1_plain_1Mbp", "gather": "2_gather_100Mbp", "fullscan":
 # {source hash: {form: {"bytes": per launch, "reads": reads per launch,
 #                       "checks": checks of the launch where it is scaled by checks}}}
 TRAFFIC_BY_SOURCE: dict[str, dict] = {
-    "df1bd25aa4ba31cc": {
-        # the dispatcher's gather by bank segment, 3.1 Gbp, 2^20 reads, 1,754,507,054 checks: prep 6,041,095,936 B
-        # read + 372,092,672 B written, scoring 52,373,728,768 + 2,488,361,216, listed reads 53,504
-        "mixed": {"bytes": 61_275_332_096, "reads": 1_048_576, "checks": 1_754_507_054},
-        # gather_kernel<5,8>, 100 Mbp, 1M reads, 74.8M checks: 598,050,048 B read + 69,929,984 B written
-        "gather": {"bytes": 667_980_032, "reads": 1_000_000},
-        # gather_kernel<5,8>, 1 Mbp, 10,000 reads, 320,000 checks: 3,024,896 B read, the output stays in L2
-        "plain": {"bytes": 3_024_896, "reads": 10_000},
+    "67909e6b32e5aa15": {
+        # the dispatcher's gather by bank segment, 3.1 Gbp, 2^20 reads, 1,754,507,054 checks: prep 6,041,421,056 B
+        # read + 372,080,128 B written, scoring 50,875,420,928 + 2,441,808,896, listed reads 57,344
+        "mixed": {"bytes": 59_730_788_352, "reads": 1_048_576, "checks": 1_754_507_054},
+        # gather_kernel<5,8>, 100 Mbp, 1M reads, 74.8M checks: 595,748,864 B read + 72,718,848 B written
+        "gather": {"bytes": 668_467_712, "reads": 1_000_000},
+        # gather_kernel<5,8>, 1 Mbp, 10,000 reads, 320,000 checks: 3,026,944 B read, the output stays in L2
+        "plain": {"bytes": 3_026_944, "reads": 10_000},
         # gather_kernel<6,8>, one 262,144-read batch of the q=6 workload, 153,942,833 checks:
-        # 47,403,621,120 B read + 161,615,104 B written
-        "batched": {"bytes": 47_565_236_224, "reads": 262_144, "checks": 153_942_833},
+        # 46,933,866,496 B read + 175,571,200 B written
+        "batched": {"bytes": 47_109_437_696, "reads": 262_144, "checks": 153_942_833},
     },
 }
 
