@@ -329,7 +329,7 @@ int grim_choose_form(const grim_bank* bank, int64_t n_reads, int64_t n_checks, i
  * consecutive gathered batches is one launch, or, with q = 5, a bank beyond
  * the L2 and rows scored many times over, three launches per 2^20 reads that
  * take the candidates segment by segment of the bank (faster for ascending
- * lists; about 300 bytes and 4 per 72 MB of bank of the library's pool for
+ * lists; about 350 bytes and 4 per 72 MB of bank of the library's pool for
  * each of those reads, and the one launch where it has none).  grim_filter,
  * grim_filter_batched and grim_filter_host never do so: for such work they are
  * the slower choice (1M reads against 3.1 Gbp, 38 ms for 23).  Reads every

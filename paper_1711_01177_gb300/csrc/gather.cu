@@ -797,9 +797,13 @@ constexpr int64_t kBlockedReads = int64_t(1) << 20;  // reads per round over the
 
 struct BlockedRead {
     int T;
-    int mode;  // 0: two planes, the upper one folded (row_sum8); 1: two planes; 2 + i: four, two of them in extra[i]
+    // 0: two planes, the upper one folded (row_sum8); 1: two planes; 2 + 2 i: three, 3 + 2 i: four, the last two in extra[i]
+    int mode;
 };
-constexpr int kExtraShare = 16;  // one read in so many may have three or four planes
+// One read in so many may have three or four planes: one in 5 of reads of 300
+// bases does, and those left over are a serial tail from HBM (3.1 Gbp, 20,000
+// reads of 300 bases, 2.60 ms at one in 16, 2.17 so; the one launch 2.30).
+constexpr int kExtraShare = 4;
 
 template <int Q>
 __global__ void __launch_bounds__(kSmallWarps * 32)
@@ -832,7 +836,7 @@ blocked_prep_kernel(const uint8_t* __restrict__ reads, const int64_t* __restrict
                     if (lane == 0) x = atomicAdd(counts + 2, 1u);
                     x = __shfl_sync(kFull, x, 0);
                     direct = x >= n_extra;
-                    mode = 2 + (int)x;
+                    mode = 2 + 2 * (int)x + (used == 4 ? 1 : 0);
                     if (!direct)
                         for (int v = lane; v < 2 * G::kRowVecs; v += 32)  // planes 2 and 3
                             extra[(size_t)x * 2 * G::kRowVecs + v] =
@@ -940,7 +944,7 @@ blocked_kernel(const uint32_t* __restrict__ bank, uint32_t n_bins32, const uint3
         auto ask_planes = [&](int which, int b) {
             ask(planes_s[warp][b], planes_in + (r0 + which) * kVecs);
             const int mode = __shfl_sync(kFull, rd.mode, which);
-            if (mode >= 2) ask(planes_s[warp][b] + kVecs, extra + (size_t)(mode - 2) * kVecs);
+            if (mode >= 2) ask(planes_s[warp][b] + kVecs, extra + (size_t)((mode - 2) >> 1) * kVecs);
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         ask_planes(i, 0);
@@ -981,7 +985,7 @@ blocked_kernel(const uint32_t* __restrict__ bank, uint32_t n_bins32, const uint3
                 score_read<Q, 2, true>(st, planes_s[warp][buf], 2, T, n_now, cand_bins + at_now, bank, n_bins32,
                                        pass + at_now, nullptr, lane, flags);
             else
-                score_read<Q, 0, true>(st, planes_s[warp][buf], 4, T, n_now, cand_bins + at_now, bank, n_bins32,
+                score_read<Q, 0, true>(st, planes_s[warp][buf], 3 + (mode & 1), T, n_now, cand_bins + at_now, bank, n_bins32,
                                        pass + at_now, nullptr, lane, flags);
             __syncwarp();
             if (!todo) break;
