@@ -59,17 +59,17 @@ SUMMARY_KEY = {"plain": "1_plain_1Mbp", "gather": "2_gather_100Mbp", "fullscan":
 # {source hash: {form: {"bytes": per launch, "reads": reads per launch,
 #                       "checks": checks of the launch where it is scaled by checks}}}
 TRAFFIC_BY_SOURCE: dict[str, dict] = {
-    "67909e6b32e5aa15": {
-        # the dispatcher's gather by bank segment, 3.1 Gbp, 2^20 reads, 1,754,507,054 checks: prep 6,041,421,056 B
-        # read + 372,080,128 B written, scoring 50,875,420,928 + 2,441,808,896, listed reads 57,344
-        "mixed": {"bytes": 59_730_788_352, "reads": 1_048_576, "checks": 1_754_507_054},
-        # gather_kernel<5,8>, 100 Mbp, 1M reads, 74.8M checks: 595,748,864 B read + 72,718,848 B written
-        "gather": {"bytes": 668_467_712, "reads": 1_000_000},
-        # gather_kernel<5,8>, 1 Mbp, 10,000 reads, 320,000 checks: 3,026,944 B read, the output stays in L2
-        "plain": {"bytes": 3_026_944, "reads": 10_000},
+    "805daae75a98a0e5": {
+        # the dispatcher's gather by bank segment, 3.1 Gbp, 2^20 reads, 1,754,507,054 checks: prep 6,040,382,208 B
+        # read + 371,548,160 B written, scoring 50,898,891,008 + 2,442,147,840, listed reads 57,088
+        "mixed": {"bytes": 59_753_026_304, "reads": 1_048_576, "checks": 1_754_507_054},
+        # gather_kernel<5,8>, 100 Mbp, 1M reads, 74.8M checks: 594,771,456 B read + 72,147,456 B written
+        "gather": {"bytes": 666_918_912, "reads": 1_000_000},
+        # gather_kernel<5,8>, 1 Mbp, 10,000 reads, 320,000 checks: 3,026,432 B read, the output stays in L2
+        "plain": {"bytes": 3_026_432, "reads": 10_000},
         # gather_kernel<6,8>, one 262,144-read batch of the q=6 workload, 153,942,833 checks:
-        # 46,933,866,496 B read + 175,571,200 B written
-        "batched": {"bytes": 47_109_437_696, "reads": 262_144, "checks": 153_942_833},
+        # 46,936,442,880 B read + 175,295,744 B written
+        "batched": {"bytes": 47_111_738_624, "reads": 262_144, "checks": 153_942_833},
     },
 }
 
